@@ -1526,20 +1526,20 @@ int grad_advance(GradJob &j, int64_t units, bool *done)
     return FWI_OK;
 }
 
-// FP64 fold of the last partial gradient and the finish into the outputs (device targets
-// of the caller or staging buffers; host copies are issued here).
+// The finish of both gradient accumulators into the outputs (device targets of the caller
+// or staging buffers; host copies are issued here).
 int grad_finish(GradJob &j, double *misfit, float *grad, double *grad64, bool *sync_needed)
 {
     fwi_model *m = j.m;
     const cudaStream_t s = j.s;
-    FWI_LAUNCH(m, launch_fold(m->g32.as<float>(), m->g64.as<double>(), j.nfield, s));
     const int64_t nphys = m->np[0] * m->np[1] * m->np[2];
     void *g32dev = nullptr, *g64dev = nullptr;
     bool g32host = false, g64host = false;
     if (grad) FWI_TRY(output_target(m, 0, grad, nphys * sizeof(float), &g32dev, &g32host));
     if (grad64) FWI_TRY(output_target(m, 1, grad64, nphys * sizeof(double), &g64dev, &g64host));
-    FWI_LAUNCH(m, launch_finish(m->g, m->nb, m->np, j.ns, m->g64.as<double>(), m->v.as<float>(),
-                                (float *)g32dev, (double *)g64dev, s));
+    ++m->launches;   // the finish is two launches
+    FWI_LAUNCH(m, launch_finish(m->g, m->nb, m->np, j.ns, m->g32.as<float>(), m->g64.as<double>(),
+                                m->v.as<float>(), (float *)g32dev, (double *)g64dev, s));
     FWI_TRY(finish_output(grad, g32dev, nphys * sizeof(float), g32host, s));
     FWI_TRY(finish_output(grad64, g64dev, nphys * sizeof(double), g64host, s));
     bool sync = g32host || g64host;

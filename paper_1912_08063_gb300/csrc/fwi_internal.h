@@ -213,9 +213,10 @@ cudaError_t launch_decode(const void *code, int64_t code_stride, const float *sc
                           int64_t n, int64_t stride, int nshots, int dtype, float *a, float *b,
                           int comps, cudaStream_t s);
 cudaError_t launch_fold(float *g32, double *g64, int64_t n, cudaStream_t s);
+// gradient from g64 + g32 (the FP32 partial needs no fold first); two launches
 cudaError_t launch_finish(const Geom &g, int nb, const int64_t np[3], int nshots,
-                          const double *g64, const float *v, float *grad32, double *grad64,
-                          cudaStream_t s);
+                          const float *g32, const double *g64, const float *v, float *grad32,
+                          double *grad64, cudaStream_t s);
 // One CTA that arms an mbarrier with an expected byte count, issues no copy and waits with
 // the step kernels' bounded wait limited to `polls`; raises bit 1 of *err when it runs
 // out (k_selftest.cu)

@@ -389,34 +389,148 @@ __global__ void k_fold(float *__restrict__ g32, double *__restrict__ g64, int64_
     }
 }
 
+// (double)x in integer instructions for zeros and normal numbers: the FP64 exponent is the
+// FP32 one plus 1023 - 127, the fraction moves up by 29 bits.
+__device__ __forceinline__ double widen(float x)
+{
+    const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
+    if (e - 1u < 254u)
+        return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))),
+                                (int)(u << 29));
+    if ((u << 1) == 0u) return __hiloint2double((int)u, 0);
+    return (double)x;   // subnormal, infinite or NaN
+}
+
+// 1 / v for FP32 v as the sum of three FP32 terms: each residual 1 - v (sum so far) is exact
+// in one FMA, so the terms leave a relative error below 2^-68, under FP64's rounding.  v
+// outside 2^-60 .. 2^60 takes the FP64 division (its residuals could underflow).
+__device__ __forceinline__ double recip(float v)
+{
+    if (!(v > 8.6736174e-19f && v < 1.1529215e18f)) return 1.0 / (double)v;
+    const float a = __frcp_rn(v);
+    const float ra = fmaf(-v, a, 1.0f), b = ra * a;
+    const float rb = fmaf(-v, b, ra), c = rb * a;
+    return widen(a) + (widen(b) + widen(c));
+}
+
+// Row `i` of k_finish's two launches: rows away from the folded faces, or on them.  Faces are
+// pz = 0 and npz - 1 and, in 3-D, py = 0 and npy - 1.
+__host__ __device__ inline int finish_inner(int n) { return n > 2 ? n - 2 : 0; }
+
+template <bool EDGE>
+__device__ __forceinline__ void finish_row(int i, int npz, int npy, bool fold_y, int &pz, int &py)
+{
+    const int iy = fold_y ? finish_inner(npy) : npy;   // rows per plane away from the faces
+    if (!EDGE) {
+        pz = 1 + i / iy;
+        py = (fold_y ? 1 : 0) + i % iy;
+        return;
+    }
+    const int zf = npz > 1 ? 2 : 1;                     // z faces: all their rows
+    if (i < zf * npy) {
+        pz = i / npy == 0 ? 0 : npz - 1;
+        py = i % npy;
+        return;
+    }
+    i -= zf * npy;                                      // y faces of the planes between
+    const int yf = npy > 1 ? 2 : 1;
+    pz = 1 + i / yf;
+    py = i % yf == 0 ? 0 : npy - 1;
+}
+
 // grad(p) = (2 / v(p)) * sum_shots sum_{computed cells c replicated from p} g_mu(c),
 // where g_mu = sum_m mu^{m+1} L u^m and mu = W nu (so dphi/dW = g_mu / W and
-// dphi/dv = 2 v dt^2 dphi/dW = 2 g_mu / v).
-// One CTA per physical row (pz, py) at a time, threads along x.
-__global__ void k_finish(Geom g, int nb, int npz, int npy, int npx, int nshots,
-                         const double *__restrict__ g64, const float *__restrict__ v,
-                         float *__restrict__ grad32, double *__restrict__ grad64)
+// dphi/dv = 2 v dt^2 dphi/dW = 2 g_mu / v); g_mu is the FP64 accumulator plus the FP32
+// partial since its last fold, so no separate last fold rewrites both.
+//
+// Bound by HBM: 12 bytes per computed cell and shot.  The sponge makes the work uneven: a
+// cell on a face gathers nb + 1 cells, one on an edge (nb + 1)^2, a corner (nb + 1)^3, times
+// the shots.  Rows (pz, py) away from the z and y faces (EDGE = false) and rows on them run
+// as two launches; a CTA takes 256 / PARTS columns of one row and PARTS groups of threads
+// share a column's list of (shot, cz, cy).  The first and last column, which also gather
+// along x, are summed by a warp (PARTS = 1) or by the whole CTA.  PARTS = 1 streams rows
+// whose list is the shots alone; 8 splits longer lists.  Measured on GB300 against one
+// thread per cell walking its whole list after a separate fold: 64 shots of 440 x 1064
+// 5128 -> 389 us, 296^3 2335 -> 551 us, 136^3 955 -> 113 us (both launches).
+//
+// The FP64 unit (about one operation per clock and SM) is what bounds it then, so FP32
+// values are widened with integer instructions (widen) and 1 / v is built from three FP32
+// terms instead of an FP64 division: 296^3 rows off the faces 1057 -> 431 us.
+template <int PARTS, bool EDGE>
+__global__ void __launch_bounds__(kThreads) k_finish(Geom g, int nb, int npz, int npy, int npx,
+                                                     int nshots, const float *__restrict__ g32,
+                                                     const double *__restrict__ g64,
+                                                     const float *__restrict__ v,
+                                                     float *__restrict__ grad32,
+                                                     double *__restrict__ grad64, int rows, int chunks)
 {
-    const int nby = (g.ndim == 3) ? nb : 0;
-    const int rows = npz * npy;
-    for (int row = blockIdx.x; row < rows; row += gridDim.x) {
-        const int pz = row / npy, py = row - pz * npy;
+    constexpr int COLS = kThreads / PARTS;
+    __shared__ double red[PARTS > 1 ? PARTS : 1][COLS];
+    const bool fold_y = g.ndim == 3;
+    const int nby = fold_y ? nb : 0;
+    const int lane = threadIdx.x % COLS, part = threadIdx.x / COLS;
+    for (int64_t w = blockIdx.x; w < (int64_t)rows * chunks; w += gridDim.x) {
+        const int row = (int)(w / chunks), chunk = (int)(w - (int64_t)row * chunks);
+        int pz, py;
+        finish_row<EDGE>(row, npz, npy, fold_y, pz, py);
         const int z0 = pz == 0 ? 0 : pz + nb, z1 = pz == npz - 1 ? pz + 2 * nb : pz + nb;
         const int y0 = py == 0 ? 0 : py + nby, y1 = py == npy - 1 ? py + 2 * nby : py + nby;
-        for (int pxx = threadIdx.x; pxx < npx; pxx += blockDim.x) {
-            const int x0 = pxx == 0 ? 0 : pxx + nb, x1 = pxx == npx - 1 ? pxx + 2 * nb : pxx + nb;
-            double acc = 0.0;
-            for (int s = 0; s < nshots; ++s) {
-                const double *gs = g64 + (int64_t)s * g.field;
-                for (int cz = z0; cz <= z1; ++cz)
-                    for (int cy = y0; cy <= y1; ++cy)
-                        for (int cx = x0; cx <= x1; ++cx)
-                            acc += gs[(int64_t)cz * g.plane + (int64_t)cy * g.px + cx];
-            }
-            const int64_t i = (int64_t)row * npx + pxx;
-            const double out = acc * 2.0 / (double)v[i];
+        const int ylen = y1 - y0 + 1, zy = (z1 - z0 + 1) * ylen, list = zy * nshots;
+        auto cell_row = [&](int e) {   // offset of row e of the list
+            const int s = e / zy, r = e - s * zy, cz = r / ylen;
+            return (int64_t)s * g.field + (int64_t)(z0 + cz) * g.plane +
+                   (int64_t)(y0 + r - cz * ylen) * g.px;
+        };
+        auto put = [&](int pxx, double acc) {
+            const int64_t i = ((int64_t)pz * npy + py) * npx + pxx;
+            const double out = acc * (2.0 * recip(v[i]));
             if (grad32) grad32[i] = (float)out;
             if (grad64) grad64[i] = out;
+        };
+        const int pxx = chunk * COLS + lane;
+        double acc = 0.0;
+        if (pxx > 0 && pxx < npx - 1) {
+#pragma unroll 4
+            for (int e = part; e < list; e += PARTS) {
+                const int64_t o = cell_row(e) + pxx + nb;
+                acc += g64[o] + widen(g32[o]);
+            }
+        }
+        if (PARTS > 1) {
+            red[part][lane] = acc;
+            __syncthreads();
+            if (part == 0) {
+#pragma unroll
+                for (int k = 1; k < PARTS; ++k) acc += red[k][lane];
+            }
+            __syncthreads();
+        }
+        if (part == 0 && pxx > 0 && pxx < npx - 1) put(pxx, acc);
+        // the first and the last column of the row
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+            const int ec = side == 0 ? 0 : npx - 1;
+            if (ec / COLS != chunk || (side == 1 && npx == 1)) continue;   // uniform per CTA
+            const int x0 = ec == 0 ? 0 : ec + nb, x1 = ec == npx - 1 ? ec + 2 * nb : ec + nb;
+            const int xl = x1 - x0 + 1;
+            const int64_t cells = (int64_t)list * xl;
+            if (PARTS == 1 && (int)(threadIdx.x >> 5) != side) continue;   // one warp each
+            const int64_t first = PARTS == 1 ? (threadIdx.x & 31) : threadIdx.x;
+            double t = 0.0;
+#pragma unroll 4
+            for (int64_t c = first; c < cells; c += PARTS == 1 ? 32 : kThreads) {
+                const int e = (int)(c / xl);
+                const int64_t o = cell_row(e) + x0 + (int)(c - (int64_t)e * xl);
+                t += g64[o] + widen(g32[o]);
+            }
+            if (PARTS == 1) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+            } else {
+                t = block_sum(t);
+                __syncthreads();   // block_sum's shared words are free for the next use
+            }
+            if (first == 0) put(ec, t);
         }
     }
 }
@@ -590,12 +704,23 @@ cudaError_t launch_fold(float *g32, double *g64, int64_t n, cudaStream_t s)
 }
 
 cudaError_t launch_finish(const Geom &g, int nb, const int64_t np[3], int nshots,
-                          const double *g64, const float *v, float *grad32, double *grad64,
-                          cudaStream_t s)
+                          const float *g32, const double *g64, const float *v, float *grad32,
+                          double *grad64, cudaStream_t s)
 {
-    const int rows = (int)(np[0] * np[1]);
-    k_finish<<<rows < 152 * 16 ? rows : 152 * 16, kThreads, 0, s>>>(
-        g, nb, (int)np[0], (int)np[1], (int)np[2], nshots, g64, v, grad32, grad64);
+    const int npz = (int)np[0], npy = (int)np[1], npx = (int)np[2];
+    const bool fold_y = g.ndim == 3;
+    const int inner = finish_inner(npz) * (fold_y ? finish_inner(npy) : npy);
+    const int edge = npz * npy - inner;
+    auto go = [&](auto kernel, int parts, int rows) {
+        if (rows < 1) return;
+        const int cols = kThreads / parts, chunks = (npx + cols - 1) / cols;
+        const int64_t work = (int64_t)rows * chunks;
+        kernel<<<(unsigned)(work < 152 * 32 ? work : 152 * 32), kThreads, 0, s>>>(
+            g, nb, npz, npy, npx, nshots, g32, g64, v, grad32, grad64, rows, chunks);
+    };
+    go(k_finish<8, true>, 8, edge);
+    if (nshots >= 8) go(k_finish<8, false>, 8, inner);
+    else go(k_finish<1, false>, 1, inner);
     return cudaGetLastError();
 }
 

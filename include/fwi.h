@@ -68,16 +68,13 @@ typedef struct {
     int32_t timing;             /* 1: bracket every time-step launch with CUDA events and
                                    accumulate kernel times (read with fwi_model_info);
                                    the call then waits for its stream at the end        */
-    int32_t temporal_blocking;  /* 1: 2-D forward calls whose shots fill the GPU advance
-                                   two time steps per pass (same results bit for bit;
-                                   measured on GB300 within 3 % of single steps: the
-                                   2-D step is latency-bound, so halving its DRAM bytes
-                                   buys nothing); 2: one-shot 2-D forward calls on grids
-                                   whose two states fit in the shared memory of one
-                                   cluster of CTAs, with node receivers on one row,
-                                   advance up to 64 steps per launch with the states on
-                                   chip (same results bit for bit); other calls run
-                                   single steps; default 0                              */
+    int32_t temporal_blocking;  /* 2: one-shot 2-D forward calls on grids whose two states
+                                   fit in the shared memory of one cluster of CTAs, with
+                                   node receivers on one row, advance up to 64 steps per
+                                   launch with the states on chip (same results bit for
+                                   bit); other calls run single steps.  0 (default) and
+                                   1: single steps (1 once advanced large batches two
+                                   steps per pass, with the same results)               */
 } fwi_opts;
 
 /* Acquisition geometry of one call: shot s has one source and nrec receivers, each a

@@ -157,7 +157,7 @@ struct fwi_model {
     // workspace
     int cap_shots = 0, cap_nrec = 0;
     DevBuf u[2], mu[2], g32, g64, traces, src_off, rec_off, inj, src_scale, maxbits, partials,
-        phi, snaps, scales, src_pts, rec_pts, step_ctr, ut[2];   // ut: spare forward states
+        phi, snaps, scales, src_pts, rec_pts, step_ctr;
     DevBuf stage_in[3], stage_out[2];
     int nslots = 0;
     size_t slot_bytes = 0;
@@ -195,9 +195,9 @@ struct fwi_model {
     };
     std::vector<MapEntry> maps;
     std::vector<MapEntry> maps2;   // 3-D maps of 2-D fields
-    // 3-D: every receiver a node of computed plane rec_fuse_z, distinct per shot: the step
-    // kernels sample and inject at them from rec_map ([shot][y][x] receiver index or -1);
-    // -1 otherwise
+    // every receiver a node of computed plane (2-D: row) rec_fuse_z, distinct per shot: the
+    // step kernels sample and inject at them from rec_map ([shot][y][x] receiver index or
+    // -1); -1 otherwise
     DevBuf rec_map;
     int rec_fuse_z = -1;
     DevBuf cl_tab;                 // one-entry table of the on-chip 2-D forward launch
@@ -222,9 +222,11 @@ struct fwi_model {
 
 namespace {
 
+// The sponge tables, each padded with zeros to a multiple of 8 floats (16-byte groups of
+// sig_x line up with groups of 4 columns; the 3-D step copies sig_z in groups of 4).
 const float *sig_z(const fwi_model *m) { return m->sig.as<float>(); }
-const float *sig_y(const fwi_model *m) { return m->sig.as<float>() + m->g.nz; }
-const float *sig_x(const fwi_model *m) { return m->sig.as<float>() + m->g.nz + m->g.ny; }
+const float *sig_y(const fwi_model *m) { return sig_z(m) + round_up(m->g.nz, 8); }
+const float *sig_x(const fwi_model *m) { return sig_y(m) + round_up(m->g.ny, 8); }
 
 int check_status(fwi_model *m)
 {
@@ -295,8 +297,7 @@ int set_velocity(fwi_model *m, const float *vp, cudaStream_t s)
     // the kernels read s = eta dt / 2 per axis
     const int nb = m->nb;
     const int ext[3] = {m->g.nz, m->g.ny, m->g.nx};
-    // 4 floats of padding: the 3-D step copies sig_z in 16-byte aligned groups of four
-    std::vector<float> sig(ext[0] + ext[1] + ext[2] + 4, 0.0f);
+    std::vector<float> sig(round_up(ext[0], 8) + round_up(ext[1], 8) + round_up(ext[2], 8), 0.0f);
     size_t base = 0;
     for (int a = 0; a < 3; ++a) {
         const bool present = !(a == 1 && m->ndim == 2);
@@ -313,7 +314,7 @@ int set_velocity(fwi_model *m, const float *vp, cudaStream_t s)
             const double eta = emax * (d / nb) * (d / nb);
             sig[base + i] = (float)(0.5 * m->dt * (nb > 0 ? eta : 0.0));
         }
-        base += ext[a];
+        base += round_up(ext[a], 8);
     }
     FWI_TRY(m->sig.ensure(sig.size() * sizeof(float)));
     FWI_CU(cudaMemcpyAsync(m->sig.p, sig.data(), sig.size() * sizeof(float),
@@ -500,7 +501,7 @@ int ensure_workspace(fwi_model *m, const fwi_acq *a, bool grad, cudaStream_t s)
         m->rec_fuse_z = -1;
         std::vector<int32_t> rmap;
         const char *fz = std::getenv("FWI_STEP3D_REC_FUSE");   // 0: separate kernels
-        if (m->ndim == 3 && !og_r && nr > 0 && !(fz && std::atoi(fz) == 0)) {
+        if (!og_r && nr > 0 && !(fz && std::atoi(fz) == 0)) {
             const int64_t plane = m->g.plane;
             const int z0 = (int)(ro[0] / plane);
             bool ok = true;
@@ -674,64 +675,48 @@ bool use_step3d(const fwi_model *m) { return m->ndim == 3; }
 
 // 3-D map [shot][z][x] of a 2-D field, cached per model like field_map's.
 int field_map2d(fwi_model *m, const void *base, int ns, int bx, CUtensorMap *out, int eb = 4,
-                int64_t stride = 0)
+                int64_t stride = 0, int bz = 1)
 {
     if (stride == 0) stride = m->g.field;
     for (const auto &e : m->maps2)
-        if (e.base == base && e.ns == ns && e.bx == bx && e.eb == eb && e.stride == stride) {
+        if (e.base == base && e.ns == ns && e.bx == bx && e.by == bz && e.eb == eb && e.stride == stride) {
             *out = e.map;
             return FWI_OK;
         }
-    fwi_model::MapEntry e{base, ns, bx, 1, eb, stride, {}};
-    if (encode_field_map2d(&e.map, base, m->g, ns, bx, eb, stride) != 0)
+    fwi_model::MapEntry e{base, ns, bx, bz, eb, stride, {}};
+    if (encode_field_map2d(&e.map, base, m->g, ns, bx, bz, eb, stride) != 0)
         return fail(FWI_ERR_CUDA, "cuTensorMapEncodeTiled failed (2-D)");
     m->maps2.push_back(e);
     *out = e.map;
     return FWI_OK;
 }
 
-// The 2-D step with TMA-staged rows, opt-in (FWI_STEP2D_TMA=1; same results bit for bit
-// as the register-streaming kernel).  Measured on GB300, 64 shots of 440 x 1064: forward
-// 0.144 against 0.103 ms, forward + store 0.150 against 0.109, reverse 0.157 against
-// 0.158 ms.  A 2-D row is 256 points per CTA: per row the staged kernel pays a CTA
-// barrier, two mbarrier round trips and five small copies (1 KB and two 16-byte halo
-// boxes), which cost more than the L1-served loads they replace; the latency they hide
-// in the reverse step only breaks even.
-bool use_step2d_tma()
+// One launch of the 2-D tile kernel (k_step2d_tile.cu).
+int step2d_tile_launch(fwi_model *m, const StepParams &p, int ns, bool img, cudaStream_t s)
 {
-    const char *e = std::getenv("FWI_STEP2D_TMA");
-    return e && std::atoi(e) != 0;
-}
-
-int step2d_tma_launch(fwi_model *m, const StepParams &p, int ns, bool img, cudaStream_t s)
-{
-    CUtensorMap maps[6];
-    FWI_TRY(field_map2d(m, p.cur, ns, 256, &maps[0]));
-    FWI_TRY(field_map2d(m, p.cur, ns, m->g.M, &maps[1]));
-    FWI_TRY(field_map2d(m, p.prev, ns, 256, &maps[2]));
-    FWI_TRY(field_map2d(m, m->W.p, 1, 256, &maps[3]));
-    if (img) {
-        FWI_TRY(field_map2d(m, p.aux, ns, 256, &maps[4], p.aux_fmt ? 2 : 4, p.aux_stride));
-        FWI_TRY(field_map2d(m, p.gacc, ns, 256, &maps[5]));
-    } else {
-        maps[4] = maps[5] = maps[2];
-    }
+    CUtensorMap map;
     StepParams q = p;
+    FWI_TRY(field_map2d(m, p.cur, ns, step2d_tile_cols() + 2 * m->g.M, &map, 4, 0,
+                        step2d_tile_rows(img) + 2 * m->g.M));
     q.err = m->d_flag;
-    FWI_CU(launch_step2d_tma(q, ns, img, maps, s));
+    // receivers handled in the epilogue: samples of a forward step that records traces (node
+    // source: off-grid source taps are added after the step, before sampling), the residual
+    // injection of a reverse step with imaging
+    q.rec_map = nullptr;
+    if (m->rec_fuse_z >= 0 && (img ? p.inj_q != nullptr : (p.rec_tr != nullptr && !m->og_src))) {
+        q.rec_map = m->rec_map.as<int>();
+        q.rec_z = m->rec_fuse_z;
+        q.nrec = m->geo_nrec;
+    }
+    FWI_CU(launch_step2d_tile(q, ns, img, map, s));
     return FWI_OK;
 }
 
-// The time step itself: in 2-D the register-streaming (or, opt-in, the TMA-staged)
-// kernel, in 3-D the TMA kernels; with `img` the reverse step that also accumulates the
-// imaging condition.
+// The time step itself: in 2-D the tile kernel, in 3-D the streaming TMA kernels; with `img`
+// the reverse step that also accumulates the imaging condition.
 int raw_step(fwi_model *m, const StepParams &p, int ns, bool img, cudaStream_t s)
 {
-    if (!use_step3d(m)) {
-        if (use_step2d_tma()) return step2d_tma_launch(m, p, ns, img, s);
-        FWI_CU(launch_step2d(p, ns, img, s));
-        return FWI_OK;
-    }
+    if (!use_step3d(m)) return step2d_tile_launch(m, p, ns, img, s);
     return step3d_launch(m, p, ns, img ? kModeAdj : kModeStep, s);
 }
 
@@ -822,7 +807,6 @@ struct FwdJob {
     float *tr = nullptr;    // device traces target (may be null)
     float *uc = nullptr, *up = nullptr;   // u^n and u^{n-1}
     int n = 0;
-    int tb_chunks = 0;      // z-chunks of the two-step pass (0: single steps only)
     int cl_size = 0;        // temporal blocking on chip: cluster size (0: off)
     // CUDA graph of one turn: g_units steps from the state buffers (g_uc, g_up), replayed
     // with the device step counter m->step_ctr (dev_n: its value as the host last set it)
@@ -858,9 +842,6 @@ int fwd_setup(FwdJob &j, fwi_model *m, int ns, int nr, const float *wav, float *
     j.uc = m->u[0].as<float>();
     j.up = m->u[1].as<float>();
     j.n = 0;
-    // 2-D batches wide enough to fill the GPU advance two steps per pass when the source
-    // is a node (off-grid source taps are added between steps)
-    j.tb_chunks = (m->og_src || m->opts.temporal_blocking != 1) ? 0 : step2d_tb2_chunks(m->g, ns);
     j.cl_size = 0;
     if (m->opts.temporal_blocking == 2 && m->ndim == 2 && ns == 1 && !m->og_src && !m->og_rec &&
         tr && !m->opts.timing) {
@@ -889,13 +870,6 @@ int fwd_setup(FwdJob &j, fwi_model *m, int ns, int nr, const float *wav, float *
             }
         }
     }
-    if (j.tb_chunks > 0) {
-        const size_t fbytes = (size_t)ns * m->g.field * sizeof(float);
-        if (m->ut[0].ensure(fbytes) != FWI_OK || m->ut[1].ensure(fbytes) != FWI_OK) {
-            cudaGetLastError();
-            j.tb_chunks = 0;   // no room for the spare states: single steps
-        }
-    }
     return FWI_OK;
 }
 
@@ -910,8 +884,8 @@ int after_forward_step(fwi_model *m, const StepParams &p, float *next, int ns, i
                                         m->W.as<float>(), sig_z(m), sig_y(m), sig_x(m),
                                         p.wavelet, m->nt, n, p.dt2, 0.0f, 0, s, p.n_dev));
     if (!traces) return FWI_OK;
-    // the 3-D step sampled the receivers itself
-    if (use_step3d(m) && m->rec_fuse_z >= 0 && !m->og_src && p.rec_tr == traces) return FWI_OK;
+    // the step sampled the receivers itself
+    if (m->rec_fuse_z >= 0 && !m->og_src && p.rec_tr == traces) return FWI_OK;
     if (m->og_rec)
         FWI_LAUNCH(m, launch_sample_pts(g, next, m->rec_pts.as<PointTaps>(), ns, nr, m->nt, n,
                                         traces, s, p.n_dev));
@@ -1023,7 +997,7 @@ int fwd_advance(FwdJob &j, int64_t units, bool *done)
     // captured graph: the buffer parity repeats after it and the step index comes from
     // the device counter
     if (units >= 2 && units <= 64 && units % 2 == 0 && m->nt - j.n >= units &&
-        !m->opts.timing && !j.g_failed && j.tb_chunks == 0) {
+        !m->opts.timing && !j.g_failed) {
         if (!j.gexec || j.g_units != units || j.g_uc != j.uc) FWI_TRY(fwd_capture(j, (int)units));
         if (j.gexec) {
             if (j.dev_n != j.n) {
@@ -1042,23 +1016,6 @@ int fwd_advance(FwdJob &j, int64_t units, bool *done)
         j.p.cur = j.uc;
         j.p.prev = j.up;
         j.p.n = j.n;
-        if (j.tb_chunks > 0 && u + 2 <= units && j.n + 2 <= m->nt) {
-            // two steps in one pass into the spare pair, which becomes the state
-            float *o1 = (j.uc == m->u[0].as<float>() || j.uc == m->u[1].as<float>())
-                            ? m->ut[0].as<float>() : m->u[0].as<float>();
-            float *o2 = (o1 == m->ut[0].as<float>()) ? m->ut[1].as<float>() : m->u[1].as<float>();
-            ++m->launches;
-            FWI_CU(launch_step2d_tb2(j.p, j.ns, o1, o2, j.tb_chunks, j.s));
-            FWI_TRY(after_forward_step(m, j.p, o1, j.ns, j.nr, j.n, j.tr, j.s));
-            StepParams p1 = j.p;
-            p1.n = j.n + 1;
-            FWI_TRY(after_forward_step(m, p1, o2, j.ns, j.nr, j.n + 1, j.tr, j.s));
-            j.up = o1;
-            j.uc = o2;
-            j.n += 2;
-            u += 2;
-            continue;
-        }
         j.p.rec_tr = j.tr;
         FWI_TRY(step_launch(m, j.p, j.ns, false, 0, j.s));
         FWI_TRY(after_forward_step(m, j.p, j.p.prev, j.ns, j.nr, j.n, j.tr, j.s));
@@ -1478,7 +1435,7 @@ int grad_advance(GradJob &j, int64_t units, bool *done)
             j.pa.n = mm;
             // node receivers on one plane: the reverse step with imaging injects the
             // residual itself
-            const bool inj_fused = img && use_step3d(m) && m->rec_fuse_z >= 0 && !m->og_rec;
+            const bool inj_fused = img && m->rec_fuse_z >= 0 && !m->og_rec;
             j.pa.inj_q = inj_fused ? j.res : nullptr;
             j.pa.inj_scale = m->inj.as<float>();
             j.pa.inj_n = mm - 1;
@@ -1617,8 +1574,7 @@ bool job_batchable(const Job *j)
 {
     if (j->kind != 0) return false;
     const fwi_model *m = j->f.m;
-    return m->ndim == 2 && j->f.ns == 1 && !m->og_src && !m->og_rec && j->f.tb_chunks == 0 &&
-           !m->opts.timing && j->f.tr != nullptr;
+    return m->ndim == 2 && j->f.ns == 1 && !m->og_src && !m->og_rec && !m->opts.timing && j->f.tr != nullptr;
 }
 
 int job_batch_entry(Job *j, Batch2dEntry *e, int zchunk)

@@ -60,9 +60,9 @@ struct StepParams {
     int64_t aux_stride;       // elements per shot
     const float *aux_scale;   // per shot at [2 s], or nullptr (scale 1)
     float *gacc;              // imaging only: gradient accumulator
-    int zchunk;               // planes per CTA along z
+    int zchunk;               // shared 2-D launch: rows per work item along z
     int nzchunks;
-    // nullable, 3-D forward step only: a checkpoint store of this step's input pair
+    // nullable, forward step only: a checkpoint store of this step's input pair
     // (cur = u^n, prev = u^{n-1}) written from the epilogue before prev is overwritten, in
     // the encode kernel's format (component a = u^n, d = u^n - u^{n-1}, or the FP32 pair)
     void *st_code;
@@ -74,10 +74,12 @@ struct StepParams {
                               // codec's scales of the new state pair)
     unsigned *err;            // TMA-staged kernels: status word, bit 1 (value 2) = a
                               // bounded wait gave up
-    // 3-D receivers sampled / residuals injected in the step's epilogue (set by the
-    // library when every receiver is a node of one plane): forward steps write
+    // receivers sampled / residuals injected in the step's epilogue (set by the library
+    // when every receiver is a node of one plane, in 2-D of one row): forward steps write
     // rec_tr[s][n][r] = u^{n+1}(rec_r); reverse steps add inj_scale[s][r] inj_q[s][inj_n][r]
     // to mu^m at the receivers (nullptr: the separate kernels do it)
+    const int *rec_map;       // 2-D: [shot][x] receiver index at row rec_z, or -1 (nullptr:
+    int rec_z, nrec;          // the step handles no receivers)
     float *rec_tr;
     const float *inj_q, *inj_scale;
     int inj_n;
@@ -113,9 +115,6 @@ cudaError_t launch_image_pts(const Geom &g, float *gacc, const void *x, int xfmt
 cudaError_t launch_gather_src_pts(const Geom &g, const float *f, const PointTaps *pts,
                                   int nshots, const float *W, float dt2, int nt, int n,
                                   float *x, cudaStream_t s);
-
-// 2-D step (k_step2d.cu); the 3-D step has its own launcher (step3d.h)
-cudaError_t launch_step2d(const StepParams &p, int nshots, bool imaging, cudaStream_t s);
 
 // The serving loop's shared 2-D forward launch: a device table of requests, each a
 // one-shot 2-D forward run with a node source and node receivers.  A tick of k steps is
@@ -154,14 +153,6 @@ int cluster2d_size(int M);
 int cluster2d_max_smem();
 cudaError_t launch_step2d_cluster(const Batch2d *tab, int M, int k, int C, int nreq, int smem,
                                   cudaStream_t s);
-// Two forward steps in one pass (2-D): from (p.cur = u^n, p.prev = u^{n-1}) write u^{n+1}
-// to out1 and u^{n+2} to out2 (neither may alias cur or prev); sources at steps n and
-// n + 1.  step2d_tb2_chunks is 0 when the batch is too small to fill the GPU (then use
-// single steps); the launcher picks its own strips and z-chunks.
-int step2d_tb2_chunks(const Geom &g, int nshots);
-cudaError_t launch_step2d_tb2(const StepParams &p, int nshots, float *out1, float *out2,
-                              int nchunks, cudaStream_t s);
-
 // ---- auxiliary kernels (k_aux.cu) ----
 cudaError_t launch_build_W(const Geom &g, int nb, const int64_t np[3], const float *v,
                            float dt, float *W, cudaStream_t s);

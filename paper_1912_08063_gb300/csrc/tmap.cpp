@@ -40,7 +40,7 @@ int encode_field_map(CUtensorMap *map, const void *base, const Geom &g, int nsho
 }
 
 int encode_field_map2d(CUtensorMap *map, const void *base, const Geom &g, int nshots, int bx,
-                       int elem_bytes, int64_t shot_stride)
+                       int bz, int elem_bytes, int64_t shot_stride)
 {
     if (elem_bytes != 4 && elem_bytes != 2) return -1;
     static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
@@ -58,7 +58,7 @@ int encode_field_map2d(CUtensorMap *map, const void *base, const Geom &g, int ns
     const cuuint64_t eb = (cuuint64_t)elem_bytes;
     const cuuint64_t dims[3] = {(cuuint64_t)g.nx, (cuuint64_t)g.nz, (cuuint64_t)nshots};
     const cuuint64_t strides[2] = {(cuuint64_t)g.px * eb, (cuuint64_t)shot_stride * eb};
-    const cuuint32_t box[3] = {(cuuint32_t)bx, 1, 1};
+    const cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)bz, 1};
     const cuuint32_t estr[3] = {1, 1, 1};
     const CUtensorMapDataType dt =
         elem_bytes == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_UINT16;

@@ -68,13 +68,12 @@ typedef struct {
     int32_t timing;             /* 1: bracket every time-step launch with CUDA events and
                                    accumulate kernel times (read with fwi_model_info);
                                    the call then waits for its stream at the end        */
-    int32_t temporal_blocking;  /* 2: one-shot 2-D forward calls on grids whose two states
-                                   fit in the shared memory of one cluster of CTAs, with
-                                   node receivers on one row, advance up to 64 steps per
-                                   launch with the states on chip (same results bit for
-                                   bit); other calls run single steps.  0 (default) and
-                                   1: single steps (1 once advanced large batches two
-                                   steps per pass, with the same results)               */
+    int32_t temporal_blocking;  /* 0 (default) and 2: 2-D calls on grids whose states fit in
+                                   the shared memory of one cluster of CTAs per shot, with
+                                   node sources and node receivers on one row, advance many
+                                   steps per launch with the states on chip (same results
+                                   bit for bit); other calls run single steps.  1: single
+                                   steps only                                            */
 } fwi_opts;
 
 /* Acquisition geometry of one call: shot s has one source and nrec receivers, each a

@@ -200,10 +200,13 @@ struct fwi_model {
     // -1); -1 otherwise
     DevBuf rec_map;
     int rec_fuse_z = -1;
-    DevBuf cl_tab;                 // one-entry table of the on-chip 2-D forward launch
-    Batch2d *cl_host = nullptr;    // its pinned staging
-    cudaEvent_t cl_up = nullptr;   // the staging's last upload finished
-    int cl_rec_z = -1, cl_rec_x0 = 0;
+    // 2-D on-chip stepping: the clusters of each size that run at once (-1: not asked yet);
+    // the schedule's per-step checkpoint entries (forward steps, then reverse
+    // steps) and slot offsets on the device, for the schedule they were uploaded for
+    int cl_active[kOnchipSizes] = {-1, -1, -1};
+    DevBuf cl_desc, cl_off;
+    std::vector<int32_t> cl_desc_host;
+    int cl_nslots = -1, cl_nt = -1;
     int resident[3] = {0, 0, 0};   // resident CTAs of the 3-D step kernel, per mode
     int resident_query[3] = {0, 0, 0};   // what the occupancy query returned (-e: error e)
     int64_t t_fwd_n = 0, t_adj_n = 0, t_st_n = 0;
@@ -799,6 +802,45 @@ int finish_output(void *user, const void *dev, size_t bytes, bool host, cudaStre
 
 namespace fwi {
 
+// CTAs per cluster with which a call on `ns` shots steps on chip, 0 if it does not: a 2-D
+// grid whose states fit the shared memory of one cluster per shot, with node sources and
+// node receivers on one row, and no more shots than clusters run at once (a second wave
+// would double the time, while the tile kernel's launches take the same few microseconds
+// for a few small shots as for one).
+int onchip_size(fwi_model *m, int ns, bool reverse)
+{
+    if (m->ndim != 2 || m->opts.temporal_blocking == 1 || m->opts.timing || m->og_src || m->og_rec ||
+        m->rec_fuse_z < 0)
+        return 0;
+    for (int i = 0; i < kOnchipSizes; ++i) {
+        const int C = kOnchipSize[i];
+        if (!onchip2d_fits(m->g, C, reverse)) continue;
+        if (m->cl_active[i] < 0) m->cl_active[i] = onchip2d_clusters(m->M, C);
+        if (ns <= m->cl_active[i]) return C;
+    }
+    return 0;
+}
+
+Onchip2d onchip_params(const fwi_model *m, const StepParams &p, int ns, int C)
+{
+    Onchip2d a{};
+    a.p = p;
+    a.p.n_dev = nullptr;
+    a.p.rec_map = m->rec_map.as<int>();
+    a.p.rec_z = m->rec_fuse_z;
+    a.p.nrec = m->geo_nrec;
+    a.C = C;
+    a.ck.ns = ns;
+    a.ck.dtype = m->opts.snap_dtype;
+    a.ck.slot_off = m->cl_off.as<int64_t>();
+    a.ck.codes = m->snaps.as<char>();
+    a.ck.half_slot = (int64_t)ns * m->g.field * (m->opts.snap_dtype == FWI_SNAP_FP32 ? 4 : 2);
+    a.ck.scales = m->scales.as<float>();
+    a.ck.maxbits = m->maxbits.as<unsigned>();
+    a.ck.flag = m->d_flag;
+    return a;
+}
+
 struct FwdJob {
     fwi_model *m = nullptr;
     cudaStream_t s = nullptr;
@@ -807,7 +849,7 @@ struct FwdJob {
     float *tr = nullptr;    // device traces target (may be null)
     float *uc = nullptr, *up = nullptr;   // u^n and u^{n-1}
     int n = 0;
-    int cl_size = 0;        // temporal blocking on chip: cluster size (0: off)
+    int onchip = 0;         // CTAs per cluster when steps run on chip (k_step2d_onchip.cu)
     // CUDA graph of one turn: g_units steps from the state buffers (g_uc, g_up), replayed
     // with the device step counter m->step_ctr (dev_n: its value as the host last set it)
     cudaGraphExec_t gexec = nullptr;
@@ -842,34 +884,7 @@ int fwd_setup(FwdJob &j, fwi_model *m, int ns, int nr, const float *wav, float *
     j.uc = m->u[0].as<float>();
     j.up = m->u[1].as<float>();
     j.n = 0;
-    j.cl_size = 0;
-    if (m->opts.temporal_blocking == 2 && m->ndim == 2 && ns == 1 && !m->og_src && !m->og_rec &&
-        tr && !m->opts.timing) {
-        // receivers on one row (sampled in the step's epilogue) and states that fit on chip
-        const int C = cluster2d_size(m->M);
-        bool ok = C > 0 && nr > 0 && m->g.nz / C > m->M &&
-                  2LL * ((m->g.nz + C - 1) / C) * m->g.px * 4 <= cluster2d_max_smem();
-        int64_t o0 = 0;
-        if (ok) {
-            o0 = node_offset(m, m->geo_rec.data());
-            const int x0 = (int)(o0 % m->g.plane);
-            ok = x0 + nr <= m->g.nx;
-            for (int r = 1; ok && r < nr; ++r) ok = node_offset(m, m->geo_rec.data() + 3 * r) == o0 + r;
-        }
-        if (ok && m->cl_tab.ensure(sizeof(Batch2d)) == FWI_OK) {
-            if (!m->cl_host) {
-                if (cudaMallocHost((void **)&m->cl_host, sizeof(Batch2d)) != cudaSuccess) {
-                    cudaGetLastError();
-                    m->cl_host = nullptr;
-                }
-            }
-            if (m->cl_host) {
-                j.cl_size = C;
-                m->cl_rec_z = (int)(o0 / m->g.plane);
-                m->cl_rec_x0 = (int)(o0 % m->g.plane);
-            }
-        }
-    }
+    j.onchip = onchip_size(m, ns, false);
     return FWI_OK;
 }
 
@@ -950,37 +965,23 @@ int fwd_capture(FwdJob &j, int units)
     return FWI_OK;
 }
 
-// Temporal blocking on chip: up to 64 steps per cluster launch (k_step2d_cluster) from a
-// one-entry table; the steps' arithmetic is the single step's.
+// Steps of one on-chip launch: a turn of the serving loop runs at least kOnchipTurn of them
+// (each launch loads and stores the states once), a direct call up to kOnchipMost.
+constexpr int64_t kOnchipTurn = 64, kOnchipMost = 1024;
+
+// Forward steps on chip; the steps' arithmetic is the single step's.
 int fwd_advance_onchip(FwdJob &j, int64_t units, bool *done)
 {
     fwi_model *m = j.m;
     for (int64_t u = 0; u < units && j.n < m->nt;) {
-        const int k = (int)std::min<int64_t>({units - u, (int64_t)(m->nt - j.n), 64});
-        if (!m->cl_up) FWI_CU(cudaEventCreateWithFlags(&m->cl_up, cudaEventDisableTiming));
-        FWI_CU(cudaEventSynchronize(m->cl_up));   // the staging is free again
-        Batch2d *h = m->cl_host;
-        h->count = 1;
-        h->total_work = h->total_rec = 0;
-        Batch2dEntry &e = h->e[0];
-        e = Batch2dEntry{};
-        e.p = j.p;
-        e.p.n_dev = nullptr;
-        e.u0 = j.uc;
-        e.u1 = j.up;
-        e.n0 = j.n;
-        e.traces = j.tr;
-        e.nrec = j.nr;
-        e.rec_off = m->rec_off.as<int64_t>();
-        e.rec_z = m->cl_rec_z;
-        e.rec_x0 = m->cl_rec_x0;
-        const int C = j.cl_size;
-        const int smem = (int)((2LL * ((m->g.nz + C - 1) / C) * m->g.px * 4 + 1023) / 1024 * 1024);
-        FWI_CU(cudaMemcpyAsync(m->cl_tab.p, h, offsetof(Batch2d, e) + sizeof(Batch2dEntry),
-                               cudaMemcpyHostToDevice, j.s));
-        FWI_CU(cudaEventRecord(m->cl_up, j.s));
-        ++m->launches;
-        FWI_CU(launch_step2d_cluster(m->cl_tab.as<Batch2d>(), m->M, k, C, 1, smem, j.s));
+        const int k = (int)std::min<int64_t>({std::max(units - u, kOnchipTurn), (int64_t)(m->nt - j.n), kOnchipMost});
+        Onchip2d a = onchip_params(m, j.p, j.ns, j.onchip);
+        a.p.rec_tr = j.tr;
+        a.u0 = j.uc;
+        a.u1 = j.up;
+        a.n0 = j.n;
+        a.k = k;
+        FWI_LAUNCH(m, launch_step2d_onchip(a, 0, j.s));
         if (k & 1) std::swap(j.uc, j.up);
         j.n += k;
         u += k;
@@ -992,7 +993,7 @@ int fwd_advance_onchip(FwdJob &j, int64_t units, bool *done)
 int fwd_advance(FwdJob &j, int64_t units, bool *done)
 {
     fwi_model *m = j.m;
-    if (j.cl_size > 0) return fwd_advance_onchip(j, units, done);
+    if (j.onchip) return fwd_advance_onchip(j, units, done);
     // a turn of an even number of steps (the serving loop's unit of work) replays one
     // captured graph: the buffer parity repeats after it and the step index comes from
     // the device counter
@@ -1047,6 +1048,7 @@ struct GradJob {
     int kdone = 0;    // forward steps already issued of the current ADVANCE action
     int aux_slot = -1;   // checkpoint the next reverse step reads u^m from in place
     int st_slot = -1, st_comps = 0;   // store the next forward step writes
+    int on_fwd = 0, on_rev = 0;   // CTAs per cluster when runs of steps go on chip
     // CUDA graphs of kGradGraphSteps plain forward steps (no checkpoint store or max-abs
     // among them), keyed by the buffer parity at their start and whether they record
     // traces, replayed with the device step counter m->step_ctr (dev_n: its value as the
@@ -1192,6 +1194,46 @@ int64_t fit_slots(Plan *m, int nt, int64_t halves)
     return lo;
 }
 
+// The schedule's checkpoint entry of every forward step (the store the step before it asks
+// for) and of every reverse step (the slot it reads u^m from), for the on-chip kernels.
+int upload_onchip_schedule(fwi_model *m, cudaStream_t s)
+{
+    if (m->cl_nslots == m->sched_nslots && m->cl_nt == m->sched_nt) return FWI_OK;
+    std::vector<int32_t> rev;
+    m->cl_desc_host.clear();
+    auto entry = [&](size_t i) {
+        const int slot = m->sched[2 * i + 1];
+        return slot | (m->slot_pair[slot] ? kOnchipPairSlot : 0) | (m->sched_comps[i] == 2 ? kOnchipPair : 0);
+    };
+    int32_t pending = -1;
+    for (size_t i = 0; i < m->sched.size() / 2; ++i) {
+        const int kind = m->sched[2 * i], arg = m->sched[2 * i + 1];
+        if (kind == 1) {
+            for (int k = 0; k < arg; ++k) {
+                m->cl_desc_host.push_back(pending);
+                pending = -1;
+            }
+        } else if (kind == 4) {
+            const bool slot = i > 0 && m->sched[2 * (i - 1)] == 3 && m->sched[2 * (i - 1) + 1] >= 0 &&
+                              m->sched_comps[i - 1] == 1;
+            rev.push_back(slot ? entry(i - 1) : -1);
+        }
+        if (kind != 1) pending = kind == 2 ? entry(i) : -1;
+    }
+    m->cl_nslots = -1;   // until the upload is issued
+    m->cl_desc_host.insert(m->cl_desc_host.end(), rev.begin(), rev.end());
+    FWI_TRY(m->cl_desc.ensure(m->cl_desc_host.size() * sizeof(int32_t)));
+    FWI_TRY(m->cl_off.ensure((m->slot_off.size() + 1) * sizeof(int64_t)));
+    FWI_CU(cudaMemcpyAsync(m->cl_desc.p, m->cl_desc_host.data(), m->cl_desc_host.size() * sizeof(int32_t),
+                           cudaMemcpyHostToDevice, s));
+    if (!m->slot_off.empty())
+        FWI_CU(cudaMemcpyAsync(m->cl_off.p, m->slot_off.data(), m->slot_off.size() * sizeof(int64_t),
+                               cudaMemcpyHostToDevice, s));
+    m->cl_nslots = m->sched_nslots;
+    m->cl_nt = m->sched_nt;
+    return FWI_OK;
+}
+
 int grad_setup(GradJob &j, fwi_model *m, const fwi_acq *acq, const float *wavelets,
                const float *d_obs, cudaStream_t s)
 {
@@ -1270,8 +1312,34 @@ int grad_setup(GradJob &j, fwi_model *m, const fwi_acq *acq, const float *wavele
     // the step kernels compute the checkpoint max-abs when asked, unless off-grid source
     // taps are added after the step (then a separate max-abs pass sees the final state)
     j.fused_max = !m->og_src;
+    j.on_fwd = onchip_size(m, ns, false);
+    j.on_rev = onchip_size(m, ns, true);
+    if (j.on_fwd || j.on_rev) FWI_TRY(upload_onchip_schedule(m, s));
     return FWI_OK;
 }
+
+// The on-chip run of forward steps that starts at action j.ia (an ADVANCE): the rest of it and
+// the (STORE, ADVANCE) pairs that follow, at most `most` steps.  Returns its steps and, in
+// *end, its last action and, in *kend, the steps of that action done by then.
+int64_t onchip_run(const GradJob &j, int64_t most, size_t *end, int *kend)
+{
+    const std::vector<int32_t> &a = j.m->sched;
+    size_t e = j.ia;
+    int64_t steps = std::min<int64_t>(a[2 * e + 1] - j.kdone, most);
+    int kd = j.kdone + (int)steps;
+    while (steps < most && kd == a[2 * e + 1] && 2 * (e + 2) < a.size() && a[2 * (e + 1)] == 2 &&
+           a[2 * (e + 2)] == 1) {
+        e += 2;
+        kd = (int)std::min<int64_t>(a[2 * e + 1], most - steps);
+        steps += kd;
+    }
+    *end = e;
+    *kend = kd;
+    return steps;
+}
+
+// Shorter runs go step by step: a launch loads and stores the states.
+constexpr int kOnchipMin = 3;
 
 int grad_advance(GradJob &j, int64_t units, bool *done)
 {
@@ -1286,6 +1354,42 @@ int grad_advance(GradJob &j, int64_t units, bool *done)
         const int kind = m->sched[2 * ia], arg = m->sched[2 * ia + 1];
         const int comps = m->sched_comps[ia];
         const bool next_store = ia + 1 < nact && m->sched[2 * (ia + 1)] == 2;
+        if (kind == 1 && j.on_fwd) {
+            size_t end;
+            int kend;
+            const int64_t steps = onchip_run(j, std::min(std::max(units - used, kOnchipTurn), kOnchipMost), &end, &kend);
+            if (steps >= kOnchipMin) {
+                Onchip2d a = onchip_params(m, j.pf, ns, j.on_fwd);
+                a.p.rec_tr = j.tr;
+                a.u0 = m->u[j.cur].as<float>();
+                a.u1 = m->u[1 - j.cur].as<float>();
+                a.n0 = (int)j.step;
+                a.k = (int)steps;
+                a.ck.rec_from = (int)std::min<int64_t>(j.recorded, nt);
+                a.ck.first_store = j.st_slot >= 0;
+                a.ck.desc = m->cl_desc.as<int32_t>() + j.nfwd;
+                FWI_LAUNCH(m, launch_step2d_onchip(a, 1, s));
+                int64_t at = j.step - j.kdone;   // the step each STORE of the run sees
+                for (size_t i = ia; i < end; i += 2) {
+                    at += m->sched[2 * i + 1];
+                    j.slot_step[m->sched[2 * (i + 1) + 1]] = at;
+                    ++j.nstore;
+                }
+                j.st_slot = -1;
+                j.step += steps;
+                j.recorded = std::max(j.recorded, j.step);
+                j.nfwd += steps;
+                used += steps;
+                if (steps & 1) j.cur = 1 - j.cur;
+                j.ia = end;
+                j.kdone = kend;
+                if (kend == m->sched[2 * end + 1]) {
+                    j.kdone = 0;
+                    ++j.ia;
+                }
+                continue;
+            }
+        }
         if (kind == 1) {   // ADVANCE (may span several turns)
             while (j.kdone < arg && used < units) {
                 // a serving turn replays a captured run of plain steps when the next
@@ -1414,6 +1518,48 @@ int grad_advance(GradJob &j, int64_t units, bool *done)
                 FWI_CU(cudaMemsetAsync(m->mu[0].p, 0, ns * j.fb, s));
                 FWI_CU(cudaMemsetAsync(m->mu[1].p, 0, ns * j.fb, s));
                 j.first_adj = false;
+            }
+            if (j.on_rev && mm < nt && j.aux_slot >= 0) {
+                // a run of reverse steps whose u^m all come from checkpoints, up to the next
+                // fold of the gradient
+                const int64_t fold = m->opts.fold_every - j.nadj % m->opts.fold_every;
+                const int64_t most = std::min({std::max(units - used, kOnchipTurn), kOnchipMost, fold});
+                int64_t steps = 1;
+                size_t end = ia;
+                while (steps < most && end + 2 < nact && m->sched[2 * (end + 1)] == 3 &&
+                       m->sched[2 * (end + 1) + 1] >= 0 && m->sched_comps[end + 1] == 1 &&
+                       m->sched[2 * (end + 2)] == 4) {
+                    end += 2;
+                    ++steps;
+                }
+                if (steps >= kOnchipMin) {
+                    Onchip2d a = onchip_params(m, j.pa, ns, j.on_rev);
+                    a.p.src_off = m->src_off.as<int64_t>();
+                    a.p.gacc = m->g32.as<float>();
+                    a.p.inj_q = j.res;
+                    a.p.inj_scale = m->inj.as<float>();
+                    a.u0 = m->mu[j.mcur].as<float>();
+                    a.u1 = m->mu[1 - j.mcur].as<float>();
+                    a.n0 = mm;
+                    a.k = (int)steps;
+                    a.ck.desc = m->cl_desc.as<int32_t>() + (m->cl_desc_host.size() - (size_t)nt) + j.nadj;
+                    FWI_LAUNCH(m, launch_step2d_onchip(a, 2, s));
+                    if (steps & 1) j.mcur = 1 - j.mcur;
+                    const int last = mm - (int)steps + 1;
+                    if (last == 1)   // mu^1 is complete: the m = 0 source term of the imaging sum
+                        FWI_LAUNCH(m, launch_src_image(g, m->mu[j.mcur].as<float>(), m->src_off.as<int64_t>(),
+                                                       m->W.as<float>(), j.pa.wavelet, j.pa.dt2, ns, nt,
+                                                       m->g64.as<double>(), s));
+                    j.aux_slot = -1;
+                    j.nadj += steps;
+                    j.nrestore += steps - 1;
+                    used += steps;
+                    j.step = last;
+                    if (j.nadj % m->opts.fold_every == 0)
+                        FWI_LAUNCH(m, launch_fold(m->g32.as<float>(), m->g64.as<double>(), j.nfield, s));
+                    j.ia = end + 1;
+                    continue;
+                }
             }
             j.pa.cur = m->mu[j.mcur].as<float>();        // mu^{m+1}
             j.pa.prev = m->mu[1 - j.mcur].as<float>();   // mu^{m+2} -> mu^m
@@ -1601,6 +1747,10 @@ int job_batch_entry(Job *j, Batch2dEntry *e, int zchunk)
     e->p.zchunk = zchunk;
     e->p.nzchunks = (m->g.nz + zchunk - 1) / zchunk;
     e->p.n_dev = nullptr;
+    e->p.rec_tr = f.tr;
+    e->p.rec_map = m->rec_fuse_z >= 0 ? m->rec_map.as<int>() : nullptr;
+    e->p.rec_z = m->rec_fuse_z;
+    e->p.nrec = f.nr;
     e->u0 = f.uc;
     e->u1 = f.up;
     e->n0 = f.n;
@@ -2024,10 +2174,9 @@ void fwi_destroy(fwi_model *m)
     m->snaps.release();
     m->scales.release();
     if (m->h_flag) cudaFreeHost(m->h_flag);
-    m->cl_tab.release();
+    m->cl_desc.release();
+    m->cl_off.release();
     m->rec_map.release();
-    if (m->cl_host) cudaFreeHost(m->cl_host);
-    if (m->cl_up) cudaEventDestroy(m->cl_up);
     for (cudaEvent_t e : m->ev) cudaEventDestroy(e);
     delete m;
 }

@@ -144,15 +144,52 @@ struct Batch2d {
 int multi2d_grid(int M);
 cudaError_t launch_step2d_multi(const Batch2d *tab, int M, int t, int grid, cudaStream_t s);
 cudaError_t launch_sample_multi(const Batch2d *tab, int t, int grid, cudaStream_t s);
-// Temporal blocking on chip: k steps of every request of the table in one launch, one
-// cluster of C CTAs per request, each CTA holding a band of rows of both states in shared
-// memory (smem bytes per CTA: 2 ceil(nz / C) px floats of the largest request).  For
-// requests with receivers on one row (rec_z >= 0) and nz / C > M.
+// ---- 2-D stepping on chip (k_step2d_onchip.cu): one cluster of C CTAs per shot, k steps per
+// launch, receivers only on one row (p.rec_map) ----
+// Schedule entry of a step: the checkpoint slot it stores to (forward) or reads u^m from
+// (reverse), -1 for none, with flags.
+constexpr int kOnchipSlot = (1 << 24) - 1;
+constexpr int kOnchipPairSlot = 1 << 24;   // the slot holds two fields per shot
+constexpr int kOnchipPair = 1 << 25;       // store the pair (u^n, u^n - u^{n-1}), not u^n alone
+// blocks of 4 x 2 points a thread may own (registers)
+constexpr int kOnchipFwdUnits = 4, kOnchipRevUnits = 2;
+// CTAs per cluster, most first: the most that leave bands of M rows
+constexpr int kOnchipSizes = 3;
+constexpr int kOnchipSize[kOnchipSizes] = {16, 8, 4};
+struct OnchipCkpt {
+    int ns;                    // shots
+    int rec_from;              // forward: record traces from this step on
+    int first_store;           // forward: desc[0] applies (else the state is stored already)
+    int dtype;                 // FWI_SNAP_*
+    const int32_t *desc;       // [k]
+    const int64_t *slot_off;   // first unit of each slot (units of half_slot bytes)
+    char *codes;
+    int64_t half_slot;
+    float *scales;             // [slots][ns][2]
+    unsigned *maxbits;         // forward with checkpoints: maxima of the last state, per shot
+    unsigned *flag;
+};
+struct Onchip2d {
+    StepParams p;              // cur, prev, n unused; rec_tr, inj_q, gacc as in a single step
+    float *u0, *u1;            // newest and older state (shots `field` apart); after k steps
+                               // they hold what k single steps would leave
+    int n0, k, C;              // first step (reverse: counts down), steps, CTAs per cluster
+    OnchipCkpt ck;
+};
 // cluster2d_size: the cluster size to use (16, else 8; 0 if clusters cannot be launched).
 int cluster2d_size(int M);
 int cluster2d_max_smem();
+// whether grid g fits on C CTAs, the shared memory per CTA it takes, and the clusters that
+// run at once
+bool onchip2d_fits(const Geom &g, int C, bool reverse);
+int onchip2d_smem(const Geom &g, int C);
+int onchip2d_clusters(int M, int C);
+// mode 0 forward, 1 forward with checkpoint stores, 2 reverse with imaging
+cudaError_t launch_step2d_onchip(const Onchip2d &a, int mode, cudaStream_t s);
+// one cluster per table entry, k steps each (fewer at the end of a run)
 cudaError_t launch_step2d_cluster(const Batch2d *tab, int M, int k, int C, int nreq, int smem,
                                   cudaStream_t s);
+
 // ---- auxiliary kernels (k_aux.cu) ----
 cudaError_t launch_build_W(const Geom &g, int nb, const int64_t np[3], const float *v,
                            float dt, float *W, cudaStream_t s);

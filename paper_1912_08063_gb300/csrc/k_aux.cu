@@ -5,6 +5,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "code16.cuh"
 #include "fwi_internal.h"
 
 namespace fwi {
@@ -205,28 +206,6 @@ __global__ void k_maxabs(const float *__restrict__ a, const float *__restrict__ 
         if (ma) atomicMax(out + 2 * s, ma);
         if (md) atomicMax(out + 2 * s + 1, md);
     }
-}
-
-// s = 2^floor(log2(T / max)) with T = 2^texp, from the bit pattern of max (exact
-// integer arithmetic); NaN for a non-finite max, 1 for an all-zero pair.
-__device__ float snap_scale(unsigned mb, int dtype)
-{
-    if (dtype == 0 || mb == 0u) return 1.0f;
-    if (mb >= 0x7f800000u) return __int_as_float(0x7fc00000);
-    const int texp = (dtype == 2) ? 14 : 0;
-    const unsigned e = mb >> 23, mant = mb & 0x7fffffu;
-    int E;
-    bool frac;
-    if (e > 0) {
-        E = (int)e - 127;
-        frac = mant != 0u;
-    } else {
-        E = (31 - __clz((int)mant)) - 149;
-        frac = (mant & (mant - 1u)) != 0u;
-    }
-    int k = texp - E - (frac ? 1 : 0);
-    k = max(-126, min(127, k));
-    return __int_as_float((k + 127) << 23);
 }
 
 // One thread per shot: the checkpoint scales from the max-abs bits (as k_encode derives

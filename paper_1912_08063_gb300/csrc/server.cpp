@@ -99,11 +99,8 @@ struct Pool {
 
 constexpr int kPoolZChunk = 128;   // most rows per work item of the multi-request step
 constexpr int kPools = 4;          // shared-launch pools per stencil radius
-// Cluster pools take grids of at most this many computed points (measured on GB300: one
-// request alone runs 4.3x / 2.3x / 1.3x faster on chip than in single steps at 128^2 /
-// 256^2 / 384^2, and no faster from about 512^2 on) and advance them by at least
-// kClusterTick steps per tick (the states stay on chip for the whole launch).
-constexpr int64_t kClusterMaxPoints = 200000;
+// Cluster pools take the grids that fit on chip and advance them by at least kClusterTick
+// steps per tick (the states stay on chip for the whole launch).
 constexpr int kClusterTick = 64;
 
 void pool_release(Pool &p)
@@ -335,9 +332,7 @@ extern "C" int fwi_serve(const fwi_request *reqs, int32_t n, const fwi_serve_opt
                 int kind = 0;
                 const int C = cl_size[ri];
                 if (C > 0 && fwi::job_batch_entry(free_slot->job, &probe, 64) == FWI_OK &&
-                    probe.rec_z >= 0 && probe.p.g.nz / C > M &&
-                    (int64_t)probe.p.g.nz * probe.p.g.px <= kClusterMaxPoints &&
-                    2LL * ((probe.p.g.nz + C - 1) / C) * probe.p.g.px * 4 <= fwi::cluster2d_max_smem())
+                    probe.p.rec_map && fwi::onchip2d_fits(probe.p.g, C, false))
                     kind = 1;
                 const int pi = (kind * 2 + ri) * kPools + (rr++ % kPools);
                 Pool &pl = pools[pi];
@@ -458,11 +453,11 @@ extern "C" int fwi_serve(const fwi_request *reqs, int32_t n, const fwi_serve_opt
                 int64_t need = 0;
                 for (int q = 0; q < h->count; ++q) {
                     const fwi::StepParams &sp = h->e[q].p;
-                    need = std::max<int64_t>(need, 2LL * ((sp.g.nz + pl.C - 1) / pl.C) * sp.g.px * 4);
+                    need = std::max<int64_t>(need, fwi::onchip2d_smem(sp.g, pl.C));
                 }
                 cudaKernelNodeParams kp = pl.params[0];
                 kp.gridDim = dim3((unsigned)(pl.C * h->count), 1, 1);
-                kp.sharedMemBytes = (unsigned)((need + 1023) / 1024 * 1024);
+                kp.sharedMemBytes = (unsigned)need;
                 if (cudaGraphExecKernelNodeSetParams(pl.exec, pl.nodes[0], &kp) != cudaSuccess) rc = FWI_ERR_CUDA;
             }
             // grids sized to this tick's work (the persistent loops cover any excess)

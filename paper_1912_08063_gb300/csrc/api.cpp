@@ -189,7 +189,7 @@ struct fwi_model {
     // TMA tensor maps of the 3-D step, keyed by buffer, shot count and box
     struct MapEntry {
         const void *base;
-        int ns, bx, by, eb;
+        int ns, bx, by, bz, eb;
         int64_t stride;
         CUtensorMap map;
     };
@@ -556,17 +556,17 @@ StepParams base_params(const fwi_model *m)
 // Tensor map of `ns` shots of a field (elements of eb bytes, shots `stride` elements
 // apart; stride 0 = the field layout), cached per model.
 int field_map(fwi_model *m, const void *base, int ns, int bx, int by, CUtensorMap *out,
-              int eb = 4, int64_t stride = 0)
+              int eb = 4, int64_t stride = 0, int bz = 1)
 {
     if (stride == 0) stride = m->g.field;
     for (const auto &e : m->maps)
-        if (e.base == base && e.ns == ns && e.bx == bx && e.by == by && e.eb == eb &&
+        if (e.base == base && e.ns == ns && e.bx == bx && e.by == by && e.bz == bz && e.eb == eb &&
             e.stride == stride) {
             *out = e.map;
             return FWI_OK;
         }
-    fwi_model::MapEntry e{base, ns, bx, by, eb, stride, {}};
-    if (encode_field_map(&e.map, base, m->g, ns, bx, by, eb, stride) != 0)
+    fwi_model::MapEntry e{base, ns, bx, by, bz, eb, stride, {}};
+    if (encode_field_map(&e.map, base, m->g, ns, bx, by, bz, eb, stride) != 0)
         return fail(FWI_ERR_CUDA, "cuTensorMapEncodeTiled failed");
     m->maps.push_back(e);
     *out = e.map;
@@ -622,11 +622,8 @@ int step3d_launch(fwi_model *m, const StepParams &p, int ns, int mode, cudaStrea
     q.sig_z = sig_z(m);
     q.err = m->d_flag;
     if (mode == kModeStep && p.st_code) mode = kModeStepStore;
-    const int TY = step3d_variant(g.M, mode).ty;
-    CUtensorMap mc, ma, mb, md, me;
-    FWI_TRY(field_map(m, p.cur, ns, 64 + 2 * g.M, TY + 2 * g.M, &mc));
-    FWI_TRY(field_map(m, p.prev, ns, 64, TY, &ma));
-    FWI_TRY(field_map(m, m->W.p, 1, 64, TY, &mb));
+    q.nshots = ns;
+    q.W = m->W.as<float>();
     q.out = p.prev;
     q.src_off = p.src_off;
     q.wavelet = p.wavelet;
@@ -634,7 +631,6 @@ int step3d_launch(fwi_model *m, const StepParams &p, int ns, int mode, cudaStrea
     q.n = p.n;
     q.n_dev = p.n_dev;
     q.dt2 = p.dt2;
-    if (mode == kModeStep && p.st_code) mode = kModeStepStore;
     if (mode == kModeStep || mode == kModeStepStore) {
         q.maxbits = p.maxbits;
         q.st_code = p.st_code;
@@ -642,12 +638,10 @@ int step3d_launch(fwi_model *m, const StepParams &p, int ns, int mode, cudaStrea
         q.st_dtype = p.st_dtype;
         q.st_comps = p.st_comps;
         q.st_cstride = p.st_cstride;
-        md = ma;
-        me = ma;
     } else {
-        FWI_TRY(field_map(m, p.aux, ns, 64, TY, &md, p.aux_fmt ? 2 : 4, p.aux_stride));
-        FWI_TRY(field_map(m, p.gacc, ns, 64, TY, &me));
         q.g = p.gacc;
+        q.aux = p.aux;
+        q.aux_stride = p.aux_stride;
         q.aux_fmt = p.aux_fmt;
         q.aux_scale = p.aux_scale;
     }
@@ -665,8 +659,26 @@ int step3d_launch(fwi_model *m, const StepParams &p, int ns, int mode, cudaStrea
         q.inj_n = p.inj_n;
     }
     ensure_resident(m);
+    if (step3d_use_brick(q, mode)) {
+        int bm[3], ba[3];
+        brick_boxes(g.M, bm, ba);
+        CUtensorMap mid, arm;
+        FWI_TRY(field_map(m, p.cur, ns, bm[0], bm[1], &mid, 4, 0, bm[2]));
+        FWI_TRY(field_map(m, p.cur, ns, ba[0], ba[1], &arm, 4, 0, ba[2]));
+        FWI_CU(launch_step3d_brick(q, mode, mid, arm, s));
+        return FWI_OK;
+    }
+    const int TY = step3d_variant(g.M, mode).ty;
+    CUtensorMap mc, ma, mb, md, me;
+    FWI_TRY(field_map(m, p.cur, ns, 64 + 2 * g.M, TY + 2 * g.M, &mc));
+    FWI_TRY(field_map(m, p.prev, ns, 64, TY, &ma));
+    FWI_TRY(field_map(m, m->W.p, 1, 64, TY, &mb));
+    md = me = ma;
+    if (mode == kModeAdj) {
+        FWI_TRY(field_map(m, p.aux, ns, 64, TY, &md, p.aux_fmt ? 2 : 4, p.aux_stride));
+        FWI_TRY(field_map(m, p.gacc, ns, 64, TY, &me));
+    }
     const int tiles = ((g.nx + 63) / 64) * ((g.ny + TY - 1) / TY);
-    q.nshots = ns;
     // z-parts in step when the streamed field is larger than the L2 (~126 MB)
     const bool in_step = (double)g.field * 4.0 * ns > 96.0 * (1 << 20);
     const int ctas = plan_persistent(q, tiles * ns, m->resident[mode], in_step);
@@ -682,11 +694,11 @@ int field_map2d(fwi_model *m, const void *base, int ns, int bx, CUtensorMap *out
 {
     if (stride == 0) stride = m->g.field;
     for (const auto &e : m->maps2)
-        if (e.base == base && e.ns == ns && e.bx == bx && e.by == bz && e.eb == eb && e.stride == stride) {
+        if (e.base == base && e.ns == ns && e.bx == bx && e.bz == bz && e.eb == eb && e.stride == stride) {
             *out = e.map;
             return FWI_OK;
         }
-    fwi_model::MapEntry e{base, ns, bx, bz, eb, stride, {}};
+    fwi_model::MapEntry e{base, ns, bx, 1, bz, eb, stride, {}};
     if (encode_field_map2d(&e.map, base, m->g, ns, bx, bz, eb, stride) != 0)
         return fail(FWI_ERR_CUDA, "cuTensorMapEncodeTiled failed (2-D)");
     m->maps2.push_back(e);

@@ -36,6 +36,9 @@ struct Step3dParams {
     int iso;                      // hx = hy = hz: the isotropic instantiation may run
     float inv_h2;                 // 1 / h^2 of an isotropic grid
     const float *sig_x, *sig_y, *sig_z;
+    const float *W;               // brick kernel: W and u^m are read without tensor maps
+    const void *aux;
+    int64_t aux_stride;           // elements per shot
     float *out;                   // the new state, over prev (in place)
     float *g;                     // kModeAdj: gradient accumulator
     const int64_t *src_off;       // may be null (kModeStep: injection; kModeAdj: g term)
@@ -120,11 +123,18 @@ Step3dKernelInfo step3d_kernel_m8(const Step3dVariant &v, int mode, bool iso = f
 Step3dKernelInfo step3d_kernel_tm8(int mode, bool iso, bool tile_g, bool half);
 Step3dKernelInfo step3d_kernel_tm4(int mode, bool iso, bool tile_g, bool half);
 
+// The brick kernel (k_step3d_brick.cu): extents (x, y, z) of its two halo boxes, and a launch
+// with the streamed field's maps of those boxes.
+void brick_boxes(int M, int (&mid)[3], int (&arm)[3]);
+bool step3d_use_brick(const Step3dParams &p, int mode);
+cudaError_t launch_step3d_brick(const Step3dParams &p, int mode, const CUtensorMap &mid,
+                                const CUtensorMap &arm, cudaStream_t s);
+
 // Encodes a 4-D tensor map over shots of a field laid out as in Geom (elements of
-// `elem_bytes` = 4 or 2, shots `shot_stride` elements apart), with box (bx, by, 1, 1) and
+// `elem_bytes` = 4 or 2, shots `shot_stride` elements apart), with box (bx, by, bz, 1) and
 // zero fill outside [0, nx) x [0, ny) x [0, nz) x [0, nshots).
 int encode_field_map(CUtensorMap *map, const void *base, const Geom &g, int nshots, int bx,
-                     int by, int elem_bytes, int64_t shot_stride);
+                     int by, int bz, int elem_bytes, int64_t shot_stride);
 
 // Segment idx (0, 1, ...) of CTA k in the persistent schedule of p over `columns` tile
 // columns: tile column *col, output planes [*z0, *z1).  Returns false past its last

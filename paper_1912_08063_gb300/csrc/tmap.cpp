@@ -7,7 +7,7 @@
 namespace fwi {
 
 int encode_field_map(CUtensorMap *map, const void *base, const Geom &g, int nshots, int bx,
-                     int by, int elem_bytes, int64_t shot_stride)
+                     int by, int bz, int elem_bytes, int64_t shot_stride)
 {
     if (elem_bytes != 4 && elem_bytes != 2) return -1;
     static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
@@ -27,7 +27,7 @@ int encode_field_map(CUtensorMap *map, const void *base, const Geom &g, int nsho
     const cuuint64_t eb = (cuuint64_t)elem_bytes;
     const cuuint64_t strides[3] = {(cuuint64_t)g.px * eb, (cuuint64_t)g.plane * eb,
                                    (cuuint64_t)shot_stride * eb};
-    const cuuint32_t box[4] = {(cuuint32_t)bx, (cuuint32_t)by, 1, 1};
+    const cuuint32_t box[4] = {(cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz, 1};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     // 16-bit codes are moved as raw 16-bit words (zero fill = +0 in either format)
     const CUtensorMapDataType dt =

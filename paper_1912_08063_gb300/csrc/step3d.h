@@ -202,7 +202,9 @@ cudaError_t launch_step2d_tile(const StepParams &p, int nshots, bool img, const 
 // column, or, with `in_step` and fewer columns than CTAs, one of S = ceil(resident /
 // columns) z-parts of a column that begin at the same z in every column: the CTAs of a
 // round then stream z in step part by part, so a tile's halo planes are still in L2 when
-// its neighbours read them (a field larger than L2 needs this).  With z-parts the planner
+// its neighbours read them (a field larger than L2 needs this).  With at least as many
+// columns as CTAs, columns are cut into parts too where whole rounds of them leave less to
+// the last, partial round.  With fewer columns than CTAs the planner
 // compares equal parts (leftovers cut over all CTAs, as one run or in pieces aligned to
 // the leftover units) with longer first parts whose leftover last parts go, in aligned
 // pieces, to the CTAs that ran a last part, and keeps the one whose busiest CTA streams

@@ -100,7 +100,44 @@ int plan_persistent(Step3dParams &p, int columns, int resident, bool in_step)
         p.rem_ctas = rem_planes > 0 ? (int)pieces : 0;
     }
     int grid = p.rounds > 0 ? resident : (p.rem_ctas > 0 ? p.rem_ctas : 1);
-    if (!in_step || columns >= resident) return grid;
+    if (!in_step) return grid;
+    if (columns >= resident) {
+        // Whole rounds of units and, for the leftover units, pieces of one length that begin
+        // at the same z in every unit, so that the CTAs of a round stream z in step and a
+        // tile's halo planes are still in L2 when its neighbours read them (one run cut over
+        // all CTAs would put them at unrelated z).  S parts per column make the leftover a
+        // smaller share at the price of S warm-ups; the S whose busiest CTA streams the
+        // fewest planes is taken.  Measured on GB300, us per launch with one run / with
+        // rounds and pieces in step: 140 x 1064 x 1064 radius 4 forward 531 / 447, store 635 /
+        // 537, reverse 721 / 661; radius 8 626 / 477, 708 / 535, 858 / 714; 296 x 552 x 1064
+        // radius 4 reverse 863 / 690; 1064^3 radius 4 forward 4218 / 3757.
+        int64_t best = -1;
+        Step3dParams b = p;
+        for (int S = 1; S <= 16 && p.nz / S >= 4 * p.M; ++S) {
+            const int len = p.nz / S, last = p.nz - (S - 1) * len;   // the last part is the longest
+            const int64_t units = (int64_t)columns * S;
+            const int rounds = (int)(units / resident), left = (int)(units - (int64_t)rounds * resident);
+            int ppu = left > 0 ? resident / left : 0;
+            while (ppu > 1 && last / ppu < 4 * p.M) --ppu;
+            const int64_t cost = (int64_t)rounds * (last + 2 * p.M) +
+                                 (left > 0 ? (last + ppu - 1) / ppu + 2 * p.M : 0);
+            if (best >= 0 && cost >= best) continue;
+            best = cost;
+            b.zparts = S;
+            b.zfirst = len;
+            b.rounds = rounds;
+            b.rem_ppu = ppu;
+            b.rem_ctas = left * ppu;
+        }
+        if (best >= 0) {
+            p.zparts = b.zparts;
+            p.zfirst = b.zfirst;
+            p.rounds = b.rounds;
+            p.rem_ppu = b.rem_ppu;
+            p.rem_ctas = b.rem_ctas;
+        }
+        return grid;
+    }
 
     const int S = (resident + columns - 1) / columns;   // (S - 1) columns < resident
     if (p.nz / S < 4 * p.M) return grid;                 // parts too thin: whole columns

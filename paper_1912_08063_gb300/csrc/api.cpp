@@ -448,7 +448,7 @@ int ensure_workspace(fwi_model *m, const fwi_acq *a, bool grad, cudaStream_t s)
     FWI_TRY(m->rec_off.ensure((size_t)ns * nr * sizeof(int64_t)));
     FWI_TRY(m->inj.ensure((size_t)ns * nr * sizeof(float)));
     FWI_TRY(m->src_scale.ensure(ns * sizeof(float)));
-    FWI_TRY(m->maxbits.ensure(2 * (ns > 64 ? ns : 64) * sizeof(unsigned)));
+    FWI_TRY(m->maxbits.ensure(4 * 2 * (ns > 64 ? ns : 64) * sizeof(unsigned)));
     FWI_TRY(m->partials.ensure(1024 * sizeof(double)));
     FWI_TRY(m->phi.ensure(sizeof(double)));
     if (grad) {
@@ -633,6 +633,8 @@ int step3d_launch(fwi_model *m, const StepParams &p, int ns, int mode, cudaStrea
     q.dt2 = p.dt2;
     if (mode == kModeStep || mode == kModeStepStore) {
         q.maxbits = p.maxbits;
+        q.max_clear = p.max_clear;
+        q.st_max = p.st_max;
         q.st_code = p.st_code;
         q.st_scale = p.st_scale;
         q.st_dtype = p.st_dtype;
@@ -848,7 +850,6 @@ Onchip2d onchip_params(const fwi_model *m, const StepParams &p, int ns, int C)
     a.ck.codes = m->snaps.as<char>();
     a.ck.half_slot = (int64_t)ns * m->g.field * (m->opts.snap_dtype == FWI_SNAP_FP32 ? 4 : 2);
     a.ck.scales = m->scales.as<float>();
-    a.ck.maxbits = m->maxbits.as<unsigned>();
     a.ck.flag = m->d_flag;
     return a;
 }
@@ -1060,6 +1061,12 @@ struct GradJob {
     int kdone = 0;    // forward steps already issued of the current ADVANCE action
     int aux_slot = -1;   // checkpoint the next reverse step reads u^m from in place
     int st_slot = -1, st_comps = 0;   // store the next forward step writes
+    // maxima of stored states: three entries used in turn behind the encode pass's own at
+    // m->maxbits.  A step that raises entry i + 1 clears i + 2, and the step after it, which
+    // stores that state, reads i + 1 for the scales: no launch of its own clears or converts
+    // them.  ring: the entry raised last.
+    int ring = 0;
+    unsigned *ring_at(int i) const { return m->maxbits.as<unsigned>() + (1 + i % 3) * 2 * (size_t)ns; }
     int on_fwd = 0, on_rev = 0;   // CTAs per cluster when runs of steps go on chip
     // CUDA graphs of kGradGraphSteps plain forward steps (no checkpoint store or max-abs
     // among them), keyed by the buffer parity at their start and whether they record
@@ -1099,8 +1106,9 @@ int grad_capture(GradJob &j, int par, bool rec)
     int rc = FWI_OK;
     StepParams p = j.pf;
     p.n_dev = m->step_ctr.as<int>();
-    p.maxbits = nullptr;
+    p.maxbits = p.max_clear = nullptr;
     p.st_code = nullptr;
+    p.st_max = nullptr;
     int cur = par;
     for (int i = 0; i < kGradGraphSteps && rc == FWI_OK; ++i) {
         p.cur = m->u[cur].as<float>();
@@ -1310,6 +1318,7 @@ int grad_setup(GradJob &j, fwi_model *m, const fwi_acq *acq, const float *wavele
     FWI_CU(cudaMemsetAsync(m->u[1].p, 0, ns * j.fb, s));
     FWI_CU(cudaMemsetAsync(m->g32.p, 0, ns * j.fb, s));
     FWI_CU(cudaMemsetAsync(m->g64.p, 0, ns * 2 * j.fb, s));
+    FWI_CU(cudaMemsetAsync(m->maxbits.p, 0, 4 * 2 * (size_t)ns * sizeof(unsigned), s));
 
     j.pf = base_params(m);
     j.pf.src_off = m->og_src ? nullptr : m->src_off.as<int64_t>();
@@ -1380,6 +1389,9 @@ int grad_advance(GradJob &j, int64_t units, bool *done)
                 a.ck.rec_from = (int)std::min<int64_t>(j.recorded, nt);
                 a.ck.first_store = j.st_slot >= 0;
                 a.ck.desc = m->cl_desc.as<int32_t>() + j.nfwd;
+                j.ring = (j.ring + 1) % 3;
+                a.ck.maxbits = j.ring_at(j.ring);
+                a.ck.max_clear = j.ring_at(j.ring + 1);
                 FWI_LAUNCH(m, launch_step2d_onchip(a, 1, s));
                 int64_t at = j.step - j.kdone;   // the step each STORE of the run sees
                 for (size_t i = ia; i < end; i += 2) {
@@ -1433,10 +1445,12 @@ int grad_advance(GradJob &j, int64_t units, bool *done)
                 j.pf.cur = m->u[j.cur].as<float>();
                 j.pf.prev = m->u[1 - j.cur].as<float>();
                 j.pf.n = (int)j.step;
-                j.pf.maxbits = nullptr;
+                j.pf.maxbits = j.pf.max_clear = nullptr;
                 j.pf.st_code = nullptr;
+                j.pf.st_max = nullptr;
                 if (j.st_slot >= 0) {   // the deferred checkpoint of this step's input pair
                     j.pf.st_code = (void *)(j.codes + m->slot_off[j.st_slot] * j.half_slot);
+                    j.pf.st_max = j.ring_at(j.ring);
                     j.pf.st_scale = m->scales.as<float>() + (size_t)j.st_slot * 2 * ns;
                     j.pf.st_dtype = m->opts.snap_dtype;
                     j.pf.st_comps = j.st_comps;
@@ -1444,8 +1458,9 @@ int grad_advance(GradJob &j, int64_t units, bool *done)
                     j.st_slot = -1;
                 }
                 if (j.fused_max && next_store && j.kdone == arg - 1) {
-                    FWI_CU(cudaMemsetAsync(m->maxbits.p, 0, 2 * ns * sizeof(unsigned), s));
-                    j.pf.maxbits = m->maxbits.as<unsigned>();
+                    j.ring = (j.ring + 1) % 3;
+                    j.pf.maxbits = j.ring_at(j.ring);
+                    j.pf.max_clear = j.ring_at(j.ring + 1);
                 }
                 const bool rec_now = j.step >= j.recorded;
                 j.pf.rec_tr = rec_now ? j.tr : nullptr;
@@ -1466,11 +1481,7 @@ int grad_advance(GradJob &j, int64_t units, bool *done)
             const bool next_adv = ia + 1 < nact && m->sched[2 * (ia + 1)] == 1;
             if (have_max && next_adv) {
                 // the next forward step reads exactly this pair: it writes the checkpoint
-                // from its epilogue with the scales derived here
-                FWI_LAUNCH(m, launch_snap_scales(m->maxbits.as<unsigned>(), ns,
-                                                 m->opts.snap_dtype,
-                                                 m->scales.as<float>() + (size_t)arg * 2 * ns,
-                                                 m->d_flag, s));
+                // and its scales
                 j.st_slot = arg;
                 j.st_comps = comps;
                 j.slot_step[arg] = j.step;
@@ -1485,7 +1496,7 @@ int grad_advance(GradJob &j, int64_t units, bool *done)
             }
             FWI_LAUNCH(m, launch_encode(m->u[j.cur].as<float>(), m->u[1 - j.cur].as<float>(),
                                         g.field, g.field, ns, m->opts.snap_dtype,
-                                        m->maxbits.as<unsigned>(),
+                                        have_max ? j.ring_at(j.ring) : m->maxbits.as<unsigned>(),
                                         (void *)(j.codes + m->slot_off[arg] * j.half_slot), slot_cstride(m, arg),
                                         m->scales.as<float>() + (size_t)arg * 2 * ns, m->d_flag,
                                         comps, s));

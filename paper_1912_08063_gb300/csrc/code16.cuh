@@ -91,4 +91,26 @@ __device__ __forceinline__ float snap_scale(unsigned mb, int dtype)
     return __int_as_float((k + 127) << 23);
 }
 
+// The scales of a checkpoint that a step writes from its epilogue, from the maxima mx of the
+// state it stores (the encode kernel's rule).
+__device__ __forceinline__ float2 store_scales(const unsigned *mx, int shot, int dtype)
+{
+    return make_float2(snap_scale(mx[2 * shot], dtype), snap_scale(mx[2 * shot + 1], dtype));
+}
+
+// What one thread does for a shot of a forward step: publishes the scales of the checkpoint
+// the step stores (raising *flag for a non-finite state) and clears the maxima that the next
+// step raises.
+__device__ __forceinline__ void store_bookkeeping(const unsigned *mx, int shot, int dtype, float *scale,
+                                                  unsigned *flag, unsigned *clear)
+{
+    if (mx) {
+        const float2 s = store_scales(mx, shot, dtype);
+        scale[2 * shot] = s.x;
+        scale[2 * shot + 1] = s.y;
+        if (mx[2 * shot] >= 0x7f800000u) atomicOr(flag, 1u);
+    }
+    if (clear) clear[2 * shot] = clear[2 * shot + 1] = 0u;
+}
+
 }  // namespace fwi

@@ -66,12 +66,14 @@ struct StepParams {
     // (cur = u^n, prev = u^{n-1}) written from the epilogue before prev is overwritten, in
     // the encode kernel's format (component a = u^n, d = u^n - u^{n-1}, or the FP32 pair)
     void *st_code;
-    const float *st_scale;    // per shot at [2s] (a) and [2s+1] (d), set by launch_snap_scales
+    const unsigned *st_max;   // the maxima of that pair, per shot at [2s] and [2s+1]: they set
+    float *st_scale;          // the scales, which the step writes here
     int st_dtype, st_comps;
     int64_t st_cstride;       // code elements per shot (both components)
     unsigned *maxbits;        // nullable, forward step only: per shot, raise [2s] / [2s+1]
                               // to the bits of max|out| / max|out - cur| (the checkpoint
                               // codec's scales of the new state pair)
+    unsigned *max_clear;      // with maxbits: the maxima that the next step will raise, cleared
     unsigned *err;            // TMA-staged kernels: status word, bit 1 (value 2) = a
                               // bounded wait gave up
     // receivers sampled / residuals injected in the step's epilogue (set by the library
@@ -167,6 +169,7 @@ struct OnchipCkpt {
     int64_t half_slot;
     float *scales;             // [slots][ns][2]
     unsigned *maxbits;         // forward with checkpoints: maxima of the last state, per shot
+    unsigned *max_clear;       // (and the maxima cleared for the step after it)
     unsigned *flag;
 };
 struct Onchip2d {
@@ -226,10 +229,6 @@ cudaError_t launch_misfit(const float *d, const float *dobs, float *r_out, int64
                           double *partials, int nblocks, double *result, unsigned *flag,
                           cudaStream_t s);
 int misfit_blocks(int64_t n);
-// per shot: scale[2s], scale[2s+1] from maxbits as the encode kernel derives them (flag
-// raised for a non-finite maximum)
-cudaError_t launch_snap_scales(const unsigned *maxbits, int nshots, int dtype, float *scale,
-                               unsigned *flag, cudaStream_t s);
 cudaError_t launch_maxabs(const float *a, const float *b, int64_t n, int64_t stride,
                           int nshots, unsigned *maxbits, cudaStream_t s);
 // comps = 2: the pair (a, b); comps = 1: a only (a checkpoint restored only for imaging)

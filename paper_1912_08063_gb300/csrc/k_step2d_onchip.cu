@@ -335,6 +335,7 @@ __device__ __forceinline__ void advance(const OnchipCkpt &a, const StepParams &p
         if (rank == 0 && tid == 0) {
             a.maxbits[2 * shot] = m.x;
             a.maxbits[2 * shot + 1] = m.y;
+            a.max_clear[2 * shot] = a.max_clear[2 * shot + 1] = 0u;
         }
     }
 }

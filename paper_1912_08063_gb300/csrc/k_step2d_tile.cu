@@ -139,11 +139,14 @@ k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUte
     if (MODE == kStore) {
         codes = (char *)p.st_code + ((int64_t)shot * p.st_cstride + off) * (p.st_dtype ? 2 : 4);
         if (p.st_dtype != 0) {
-            sca = p.st_scale[2 * shot];
-            scd = p.st_scale[2 * shot + 1];
+            const float2 sc = store_scales(p.st_max, shot, p.st_dtype);
+            sca = sc.x;
+            scd = sc.y;
         }
     }
     const float ainv = (MODE == kImg && p.aux_scale) ? 1.0f / p.aux_scale[2 * shot] : 1.0f;
+    if (MODE != kImg && threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0)
+        store_bookkeeping(p.st_max, shot, p.st_dtype, p.st_scale, p.err, p.max_clear);
     __syncthreads();   // the barrier is initialised
     const bool ok = mbar_wait(&bar, 0);
     if (!ok) {

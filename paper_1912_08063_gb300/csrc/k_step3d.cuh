@@ -591,8 +591,9 @@ __device__ __forceinline__ void run_segment(Ctx<C, MODE> &c, int col, int z0, in
     if (c.tid == 0 && MODE == kModeAdj)
         *(float *)c.ainv = p.aux_scale ? 1.0f / p.aux_scale[2 * c.shot] : 1.0f;
     if (c.tid == 0 && MODE == kModeStepStore) {
-        ((float *)c.sts)[0] = p.st_scale[2 * c.shot];
-        ((float *)c.sts)[1] = p.st_scale[2 * c.shot + 1];
+        const float2 sc = store_scales(p.st_max, c.shot, p.st_dtype);
+        ((float *)c.sts)[0] = sc.x;
+        ((float *)c.sts)[1] = sc.y;
     }
     // every thread is past the previous segment: its stages may be refilled
     __syncthreads();
@@ -684,6 +685,9 @@ k_step3d_tma(const __grid_constant__ Step3dParams p, const __grid_constant__ CUt
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
 
+    if (MODE != kModeAdj && blockIdx.x == 0 && c.tid == 0)
+        for (int k = 0; k < p.nshots; ++k)
+            store_bookkeeping(p.st_max, k, p.st_dtype, p.st_scale, p.err, p.max_clear);
     const int tiles_x = (p.nx + C::TX - 1) / C::TX;
     const int tiles = tiles_x * ((p.ny + C::TY - 1) / C::TY);
     walk_schedule(p, tiles * p.nshots, c.abort_flag,

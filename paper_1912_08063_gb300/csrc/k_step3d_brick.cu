@@ -224,10 +224,13 @@ k_step3d_brick(const __grid_constant__ Step3dParams p, const __grid_constant__ C
     }
     float sca = 1.0f, scd = 1.0f;
     if (MODE == kModeStepStore) {
-        sca = p.st_scale[2 * shot];
-        scd = p.st_scale[2 * shot + 1];
+        const float2 sc = store_scales(p.st_max, shot, p.st_dtype);
+        sca = sc.x;
+        scd = sc.y;
     }
     const float ainv = (MODE == kModeAdj && p.aux_scale) ? 1.0f / p.aux_scale[2 * shot] : 1.0f;
+    if (MODE != kModeAdj && tid == 0 && blockIdx.x == 0 && blockIdx.y == 0 && bz == 0)
+        store_bookkeeping(p.st_max, shot, p.st_dtype, p.st_scale, p.err, p.max_clear);
     __syncthreads();   // the barrier is initialised
     if (!mbar_wait(&bar, 0)) {
         // a bounded wait gave up: report, then give the copies a bounded chance to land

@@ -51,12 +51,14 @@ struct Step3dParams {
                                   // checkpoint codes
     const float *aux_scale;       // kModeAdj with codes: per shot at [2 s] (u = code / scale)
     void *st_code;                // kModeStep, nullable: checkpoint of the input pair (c, prev)
-    const float *st_scale;        //   written from the epilogue (see StepParams)
+    const unsigned *st_max;       //   written from the epilogue (see StepParams)
+    float *st_scale;
     int st_dtype, st_comps;
     int64_t st_cstride;
     unsigned *maxbits;            // kModeStep, nullable: per shot, raise [2s] to the bits of
                                   // max|out| and [2s+1] to max|out - c| (the checkpoint
                                   // codec's scales of the new state pair)
+    unsigned *max_clear;          // with maxbits: maxima cleared for the next step
     // receivers handled in the epilogue (rec_map nullable): every receiver is the node
     // (rec_z, y, x) with rec_map[shot][y][x] = its index (-1 elsewhere); forward modes
     // write rec_tr[shot][n][r] = out, the reverse mode adds

@@ -33,6 +33,7 @@
 #include "code16.cuh"
 #include "fwi_internal.h"
 #include "k_step3d.cuh"
+#include "pdl.cuh"
 #include "step2d_math.cuh"
 
 namespace fwi {
@@ -75,12 +76,11 @@ k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUte
     __shared__ __align__(8) uint64_t bar;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int shot = blockIdx.z, nz = p.g.nz, nx = p.g.nx;
+    pdl_next();
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_expect_tx(&bar, SX * SZ * 4);
-        tma_tile(&tile[0][0], &map, blockIdx.x * kTileX - M, blockIdx.y * TZ - M, shot, &bar);
     }
     const int x0 = blockIdx.x * kTileX + 4 * lane, zr = blockIdx.y * TZ + warp * RZ;
     const bool xin = x0 < nx;
@@ -97,10 +97,21 @@ k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUte
     float *__restrict__ gp = MODE == kImg ? p.gacc + sb : nullptr;
     const char *__restrict__ up =
         MODE == kImg ? (const char *)p.aux + ((int64_t)shot * p.aux_stride + off) * (afmt ? 2 : 4) : nullptr;
+    float sz[RZ];
+#pragma unroll
+    for (int r = 0; r < RZ; ++r) {
+        Wv[r] = r < left ? __ldg((const float4 *)(Wp + r * plane)) : zero4;
+        sz[r] = __ldg(p.sig_z + min(zr + r, nz - 1));
+    }
+    const float4 sx4 = xin ? __ldg((const float4 *)(p.sig_x + x0)) : zero4;   // padded with zeros
+    pdl_wait();
+    if (threadIdx.x == 0) {
+        mbar_expect_tx(&bar, SX * SZ * 4);
+        tma_tile(&tile[0][0], &map, blockIdx.x * kTileX - M, blockIdx.y * TZ - M, shot, &bar);
+    }
 #pragma unroll
     for (int r = 0; r < RZ; ++r) {
         pv[r] = r < left ? *(const float4 *)(prev + r * plane) : zero4;
-        Wv[r] = r < left ? __ldg((const float4 *)(Wp + r * plane)) : zero4;
         if (MODE == kImg) {
             gv[r] = r < left ? *(const float4 *)(gp + r * plane) : zero4;
             ur[r] = make_uint4(0u, 0u, 0u, 0u);
@@ -115,10 +126,6 @@ k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUte
             }
         }
     }
-    const float4 sx4 = xin ? __ldg((const float4 *)(p.sig_x + x0)) : zero4;   // padded with zeros
-    float sz[RZ];
-#pragma unroll
-    for (int r = 0; r < RZ; ++r) sz[r] = __ldg(p.sig_z + min(zr + r, nz - 1));
     const int n = (p.n_dev ? *p.n_dev : 0) + p.n;
     int src_r = -1, src_e = 0;
     float srcv = 0.0f;
@@ -239,8 +246,7 @@ cudaError_t go(const StepParams &p, int nshots, const CUtensorMap &map, cudaStre
 {
     constexpr int TZ = kWarps * tile_rz(MODE);
     const dim3 grid((p.g.nx + kTileX - 1) / kTileX, (p.g.nz + TZ - 1) / TZ, nshots);
-    k_step2d_tile<M, MODE><<<grid, 32 * kWarps, 0, s>>>(p, map);
-    return cudaGetLastError();
+    return launch_pdl(k_step2d_tile<M, MODE>, grid, dim3(32 * kWarps), 0, s, p, map);
 }
 
 }  // namespace

@@ -7,6 +7,7 @@
 
 #include <algorithm>
 
+#include "pdl.cuh"
 #include "step3d.h"
 
 namespace fwi {
@@ -139,6 +140,11 @@ cudaError_t launch_step3d_tma(const Step3dParams &p, int mode, int ctas,
     const cudaError_t e = prepare_kernel(k);
     if (e != cudaSuccess) return e;
     if (ctas < 1) return cudaErrorInvalidValue;
+    // Programmatic launches at radius 4 (1024^3 forward call 379 -> 349 ms, 256^3 gradient 108.4
+    // -> 107.9 ms) and plain ones at radius 8, whose reverse step loses what it gains and more
+    // (512^3 gradient 375 ms plain, 395 with a programmatic reverse step, 377 and 379 with
+    // programmatic forward and storing steps).
+    if (p.M == 4) return launch_pdl(k.fn, dim3(ctas), dim3(k.threads), k.smem, s, p, mc, ma, mb, md, me);
     k.fn<<<ctas, k.threads, k.smem, s>>>(p, mc, ma, mb, md, me);
     return cudaGetLastError();
 }

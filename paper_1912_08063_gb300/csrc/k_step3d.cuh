@@ -53,6 +53,7 @@
 
 #include "code16.cuh"
 #include "fwi_internal.h"
+#include "pdl.cuh"
 #include "step3d.h"
 
 namespace fwi {
@@ -685,6 +686,8 @@ k_step3d_tma(const __grid_constant__ Step3dParams p, const __grid_constant__ CUt
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
 
+    pdl_next();
+    pdl_wait();
     if (MODE != kModeAdj && blockIdx.x == 0 && c.tid == 0)
         for (int k = 0; k < p.nshots; ++k)
             store_bookkeeping(p.st_max, k, p.st_dtype, p.st_scale, p.err, p.max_clear);

@@ -30,6 +30,7 @@
 #include <cstdlib>
 
 #include "k_step3d.cuh"
+#include "pdl.cuh"
 
 namespace fwi {
 namespace {
@@ -160,14 +161,11 @@ k_step3d_brick(const __grid_constant__ Step3dParams p, const __grid_constant__ C
     const int tid = threadIdx.x, tx = tid & 7, ty = (tid >> 3) & 3, tz = tid >> 5;
     const int shot = blockIdx.z / tiles_z, bz = blockIdx.z - shot * tiles_z;
     const int X0 = blockIdx.x * TX, Y0 = blockIdx.y * TY, Z0 = bz * TZ;
+    pdl_next();
     if (tid == 0) {
         mbar_init(&bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_expect_tx(&bar, (C::MID + 2 * C::ARM) * 4);
-        tma_load4(mid, &map_mid, X0 - M, Y0 - M, Z0, shot, &bar);
-        tma_load4(zlo, &map_arm, X0, Y0, Z0 - M, shot, &bar);
-        tma_load4(zhi, &map_arm, X0, Y0, Z0 + TZ, shot, &bar);
     }
     const int x0 = X0 + 4 * tx, y0 = Y0 + RY * ty, zb = Z0 + RZ * tz;
     const int px = p.px;
@@ -184,9 +182,27 @@ k_step3d_brick(const __grid_constant__ Step3dParams p, const __grid_constant__ C
 #pragma unroll
         for (int r = 0; r < RY; ++r) {
             ok[i][r] = x0 < p.nx && y0 + r < p.ny && zb + i < p.nz;
+            Wv[i][r] = ok[i][r] ? __ldg((const float4 *)(p.W + off + (int64_t)i * p.plane + r * px)) : zero4;
+        }
+    const float4 sx = x0 < p.nx ? __ldg((const float4 *)(p.sig_x + x0)) : zero4;   // padded with zeros
+    float syr[RY], szr[RZ];
+#pragma unroll
+    for (int r = 0; r < RY; ++r) syr[r] = y0 + r < p.ny ? p.sig_y[y0 + r] : 0.0f;
+#pragma unroll
+    for (int i = 0; i < RZ; ++i) szr[i] = zb + i < p.nz ? p.sig_z[zb + i] : 0.0f;
+    pdl_wait();
+    if (tid == 0) {
+        mbar_expect_tx(&bar, (C::MID + 2 * C::ARM) * 4);
+        tma_load4(mid, &map_mid, X0 - M, Y0 - M, Z0, shot, &bar);
+        tma_load4(zlo, &map_arm, X0, Y0, Z0 - M, shot, &bar);
+        tma_load4(zhi, &map_arm, X0, Y0, Z0 + TZ, shot, &bar);
+    }
+#pragma unroll
+    for (int i = 0; i < RZ; ++i)
+#pragma unroll
+        for (int r = 0; r < RY; ++r) {
             const int64_t o = (int64_t)i * p.plane + r * px;
             pv[i][r] = ok[i][r] ? *(const float4 *)(out + o) : zero4;
-            Wv[i][r] = ok[i][r] ? __ldg((const float4 *)(p.W + off + o)) : zero4;
             if (MODE == kModeAdj) {
                 gv[i][r] = ok[i][r] ? *(const float4 *)(p.g + sb + o) : zero4;
                 ur[i][r] = make_uint4(0u, 0u, 0u, 0u);
@@ -202,12 +218,6 @@ k_step3d_brick(const __grid_constant__ Step3dParams p, const __grid_constant__ C
                 }
             }
         }
-    const float4 sx = x0 < p.nx ? __ldg((const float4 *)(p.sig_x + x0)) : zero4;   // padded with zeros
-    float syr[RY], szr[RZ];
-#pragma unroll
-    for (int r = 0; r < RY; ++r) syr[r] = y0 + r < p.ny ? p.sig_y[y0 + r] : 0.0f;
-#pragma unroll
-    for (int i = 0; i < RZ; ++i) szr[i] = zb + i < p.nz ? p.sig_z[zb + i] : 0.0f;
     const int n = (p.n_dev ? *p.n_dev : 0) + p.n;
     int src_i = -1, src_r = 0, src_e = 0;
     float srcv = 0.0f;
@@ -412,8 +422,7 @@ cudaError_t go(const Step3dParams &p, int nshots, const CUtensorMap &mid, const 
     if (e != cudaSuccess) return e;
     const int tz = (p.nz + C::TZ - 1) / C::TZ;
     const dim3 grid((p.nx + C::TX - 1) / C::TX, (p.ny + C::TY - 1) / C::TY, tz * nshots);
-    fn<<<grid, C::NT, C::SMEM, s>>>(p, mid, arm, tz);
-    return cudaGetLastError();
+    return launch_pdl(fn, grid, dim3(C::NT), C::SMEM, s, p, mid, arm, tz);
 }
 
 template <int M, bool ISO>

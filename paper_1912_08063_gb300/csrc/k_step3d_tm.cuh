@@ -35,6 +35,7 @@
 #pragma once
 
 #include "k_step3d.cuh"
+#include "pdl.cuh"
 
 namespace fwi {
 namespace s3tm {
@@ -694,6 +695,7 @@ k_step3d_tm(const __grid_constant__ Step3dParams p, const __grid_constant__ CUte
     c.h_issued = c.p_issued = 0;
     c.mxa = c.mxd = 0.0f;
 
+    pdl_next();
     const int warp = c.tid >> 5;
     if (warp == 0) tmem_alloc(tbase, C::TCOLS);
     if (c.tid == 0) {
@@ -712,6 +714,7 @@ k_step3d_tm(const __grid_constant__ Step3dParams p, const __grid_constant__ CUte
         c.tpart = c.traw + C::RING;
     }
 
+    pdl_wait();
     if (MODE != kModeAdj && blockIdx.x == 0 && c.tid == 0)
         for (int k = 0; k < p.nshots; ++k)
             store_bookkeeping(p.st_max, k, p.st_dtype, p.st_scale, p.err, p.max_clear);

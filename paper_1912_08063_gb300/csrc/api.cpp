@@ -626,6 +626,7 @@ int step3d_launch(fwi_model *m, const StepParams &p, int ns, int mode, cudaStrea
     q.W = m->W.as<float>();
     q.out = p.prev;
     q.src_off = p.src_off;
+    q.src_pts = p.src_pts;
     q.wavelet = p.wavelet;
     q.nt = p.nt;
     q.n = p.n;
@@ -651,7 +652,7 @@ int step3d_launch(fwi_model *m, const StepParams &p, int ns, int mode, cudaStrea
     // (node source: off-grid source taps are added after the step, before sampling), the
     // residual injection of a reverse step with imaging
     if (m->rec_fuse_z >= 0 &&
-        (mode == kModeAdj ? p.inj_q != nullptr : (p.rec_tr != nullptr && !m->og_src))) {
+        (mode == kModeAdj ? p.inj_q != nullptr : (p.rec_tr != nullptr && (!m->og_src || p.src_pts)))) {
         q.rec_map = m->rec_map.as<int>();
         q.rec_z = m->rec_fuse_z;
         q.nrec = m->geo_nrec;
@@ -720,7 +721,8 @@ int step2d_tile_launch(fwi_model *m, const StepParams &p, int ns, bool img, cuda
     // source: off-grid source taps are added after the step, before sampling), the residual
     // injection of a reverse step with imaging
     q.rec_map = nullptr;
-    if (m->rec_fuse_z >= 0 && (img ? p.inj_q != nullptr : (p.rec_tr != nullptr && !m->og_src))) {
+    if (m->rec_fuse_z >= 0 &&
+        (img ? p.inj_q != nullptr : (p.rec_tr != nullptr && (!m->og_src || p.src_pts)))) {
         q.rec_map = m->rec_map.as<int>();
         q.rec_z = m->rec_fuse_z;
         q.nrec = m->geo_nrec;
@@ -879,6 +881,23 @@ struct FwdJob {
     }
 };
 
+// Off-grid source taps of a forward step that adds them itself (the 2-D tile kernel and the
+// 3-D brick kernel, in both of their forward modes), else nullptr: injected after each step.
+const PointTaps *step_taps(const fwi_model *m, int ns)
+{
+    if (!m->og_src) return nullptr;
+    if (m->ndim == 3) {
+        Step3dParams q{};
+        q.M = m->g.M;
+        q.nx = m->g.nx;
+        q.ny = m->g.ny;
+        q.nz = m->g.nz;
+        q.nshots = ns;
+        if (!step3d_use_brick(q, kModeStep) || !step3d_use_brick(q, kModeStepStore)) return nullptr;
+    }
+    return m->src_pts.as<PointTaps>();
+}
+
 int fwd_setup(FwdJob &j, fwi_model *m, int ns, int nr, const float *wav, float *tr,
               cudaStream_t s)
 {
@@ -891,8 +910,8 @@ int fwd_setup(FwdJob &j, fwi_model *m, int ns, int nr, const float *wav, float *
     FWI_CU(cudaMemsetAsync(m->u[0].p, 0, ns * fb, s));
     FWI_CU(cudaMemsetAsync(m->u[1].p, 0, ns * fb, s));
     j.p = base_params(m);
-    // an on-grid source is injected inside the step; off-grid taps right after it
     j.p.src_off = m->og_src ? nullptr : m->src_off.as<int64_t>();
+    j.p.src_pts = step_taps(m, ns);
     j.p.wavelet = wav;
     j.uc = m->u[0].as<float>();
     j.up = m->u[1].as<float>();
@@ -907,13 +926,13 @@ int after_forward_step(fwi_model *m, const StepParams &p, float *next, int ns, i
                        float *traces, cudaStream_t s)
 {
     const Geom &g = m->g;
-    if (m->og_src)
+    if (m->og_src && !p.src_pts)
         FWI_LAUNCH(m, launch_inject_pts(g, next, m->src_pts.as<PointTaps>(), ns, 1,
                                         m->W.as<float>(), sig_z(m), sig_y(m), sig_x(m),
                                         p.wavelet, m->nt, n, p.dt2, 0.0f, 0, s, p.n_dev));
     if (!traces) return FWI_OK;
     // the step sampled the receivers itself
-    if (m->rec_fuse_z >= 0 && !m->og_src && p.rec_tr == traces) return FWI_OK;
+    if (m->rec_fuse_z >= 0 && (!m->og_src || p.src_pts) && p.rec_tr == traces) return FWI_OK;
     if (m->og_rec)
         FWI_LAUNCH(m, launch_sample_pts(g, next, m->rec_pts.as<PointTaps>(), ns, nr, m->nt, n,
                                         traces, s, p.n_dev));
@@ -1322,6 +1341,7 @@ int grad_setup(GradJob &j, fwi_model *m, const fwi_acq *acq, const float *wavele
 
     j.pf = base_params(m);
     j.pf.src_off = m->og_src ? nullptr : m->src_off.as<int64_t>();
+    j.pf.src_pts = step_taps(m, ns);
     j.pf.wavelet = (const float *)wav;
     j.pa = base_params(m);   // reverse sweep: receivers injected after each step; the
                              // wavelet enters only the imaging term at the source point
@@ -1332,7 +1352,7 @@ int grad_setup(GradJob &j, fwi_model *m, const fwi_acq *acq, const float *wavele
     j.codes = m->snaps.as<char>();
     // the step kernels compute the checkpoint max-abs when asked, unless off-grid source
     // taps are added after the step (then a separate max-abs pass sees the final state)
-    j.fused_max = !m->og_src;
+    j.fused_max = !m->og_src || j.pf.src_pts;
     j.on_fwd = onchip_size(m, ns, false);
     j.on_rev = onchip_size(m, ns, true);
     if (j.on_fwd || j.on_rev) FWI_TRY(upload_onchip_schedule(m, s));
@@ -1609,33 +1629,42 @@ int grad_advance(GradJob &j, int64_t units, bool *done)
             j.pa.inj_scale = m->inj.as<float>();
             j.pa.inj_n = mm - 1;
             FWI_TRY(step_launch(m, j.pa, ns, img, 1, s));
-            if (img && m->og_src)   // source term of the imaging sum at the source taps
-                FWI_LAUNCH(m, launch_image_pts(g, m->g32.as<float>(), j.pa.cur, 0, g.field,
-                                               nullptr, m->src_pts.as<PointTaps>(), ns, 1,
-                                               m->W.as<float>(), j.pa.wavelet, nt, mm,
-                                               j.pa.dt2, 0, s));
-            if (m->og_rec) {
-                // receiver term of the imaging sum (u^m at the taps), then the injection
-                FWI_LAUNCH(m, launch_image_pts(g, m->g32.as<float>(), j.pa.aux, j.pa.aux_fmt,
-                                               j.pa.aux_stride, j.pa.aux_scale,
-                                               m->rec_pts.as<PointTaps>(), ns * nr, nr,
-                                               m->W.as<float>(), j.res, nt, mm - 1, j.pa.dt2,
-                                               1, s));
-                FWI_LAUNCH(m, launch_inject_pts(g, j.pa.prev, m->rec_pts.as<PointTaps>(),
-                                                ns * nr, nr, m->W.as<float>(), sig_z(m),
-                                                sig_y(m), sig_x(m), j.res, nt, mm - 1,
-                                                j.pa.dt2, 2.0f, 1, s));
-            } else if (!inj_fused) {
+            AdjointPts ap{};
+            ap.nt = nt;
+            ap.m = mm;
+            ap.rec = m->rec_pts.as<PointTaps>();
+            ap.src = m->src_pts.as<PointTaps>();
+            ap.g = m->g32.as<float>();
+            ap.mu = j.pa.prev;
+            ap.mu1 = j.pa.cur;
+            ap.x = j.pa.aux;
+            ap.xfmt = j.pa.aux_fmt;
+            ap.xstride = j.pa.aux_stride;
+            ap.xscale = j.pa.aux_scale;
+            ap.W = m->W.as<float>();
+            ap.sz = sig_z(m);
+            ap.sy = sig_y(m);
+            ap.sx = sig_x(m);
+            ap.res = j.res;
+            ap.wav = j.pa.wavelet;
+            ap.dt2 = j.pa.dt2;
+            ap.factor = 2.0f;
+            ap.per_shot = nr;
+            ap.npts = m->og_rec ? ns * nr : 0;          // receivers: image term and injection
+            ap.nsrc = img && m->og_src ? ns : 0;        // sources: image term
+            if (ap.npts + ap.nsrc > 0) FWI_LAUNCH(m, launch_adjoint_pts(g, ap, s));
+            if (!m->og_rec && !inj_fused) {
                 FWI_LAUNCH(m, launch_inject(g, j.pa.prev, m->rec_off.as<int64_t>(),
                                             m->inj.as<float>(), j.res, ns, nr, nt, mm - 1, s));
             }
             if (mm == 1) {   // mu^1 is complete: the m = 0 source term of the imaging sum
-                if (m->og_src)
-                    FWI_LAUNCH(m, launch_image_pts(g, m->g32.as<float>(), j.pa.prev, 0, g.field,
-                                                   nullptr, m->src_pts.as<PointTaps>(), ns, 1,
-                                                   m->W.as<float>(), j.pa.wavelet, nt, 0,
-                                                   j.pa.dt2, 0, s));
-                else
+                if (m->og_src) {
+                    ap.m = 0;
+                    ap.mu1 = j.pa.prev;
+                    ap.npts = 0;
+                    ap.nsrc = ns;
+                    FWI_LAUNCH(m, launch_adjoint_pts(g, ap, s));
+                } else
                     FWI_LAUNCH(m, launch_src_image(g, j.pa.prev, m->src_off.as<int64_t>(),
                                                    m->W.as<float>(), j.pa.wavelet, j.pa.dt2, ns,
                                                    nt, m->g64.as<double>(), s));

@@ -47,6 +47,8 @@ struct StepParams {
     const float *W;
     const float *sig_z, *sig_y, *sig_x;
     const int64_t *src_off;   // [nshots] offsets within a shot's field, or nullptr
+    const struct PointTaps *src_pts;   // off-grid sources added by the step itself: [nshots] taps, or
+                              // nullptr (2-D and the 3-D brick kernel, forward modes)
     const float *wavelet;     // [nshots][nt]
     int nt, n;
     const int *n_dev;         // nullable: the step index is *n_dev + n (a captured CUDA graph
@@ -107,12 +109,20 @@ cudaError_t launch_inject_pts(const Geom &g, float *f, const PointTaps *pts, int
                               const float *sig_y, const float *sig_x, const float *q, int nt,
                               int n, float dt2, float factor, int kind, cudaStream_t s,
                               const int *n_dev = nullptr);
-// transposed-imaging point terms: kind 0 g -= dt^2 q[s][n] wt x / W (x = mu^{m+1});
-// kind 1 g += 2 wt x q[s][n][r] (x = u^m as FP32 or a 16-bit code, see StepParams::aux)
-cudaError_t launch_image_pts(const Geom &g, float *gacc, const void *x, int xfmt,
-                             int64_t xstride, const float *xscale, const PointTaps *pts,
-                             int npts, int per_shot, const float *W, const float *q, int nt,
-                             int n, float dt2, int kind, cudaStream_t s);
+// The point work of reverse step m: receivers' image terms and injections, sources' image terms
+struct AdjointPts {
+    int npts, per_shot, nsrc, nt, m;   // receivers of all shots, per shot, sources, steps
+    const PointTaps *rec, *src;
+    float *g, *mu;                     // gradient accumulator, mu^m
+    const float *mu1;                  // mu^{m+1} (sources)
+    const void *x;                     // u^m as an FP32 field or a 16-bit code (StepParams::aux)
+    int xfmt;
+    int64_t xstride;
+    const float *xscale;
+    const float *W, *sz, *sy, *sx, *res, *wav;
+    float dt2, factor;
+};
+cudaError_t launch_adjoint_pts(const Geom &g, const AdjointPts &a, cudaStream_t s);
 // x[s][n] = dt^2 sum_t wt f[t] / W[t]
 cudaError_t launch_gather_src_pts(const Geom &g, const float *f, const PointTaps *pts,
                                   int nshots, const float *W, float dt2, int nt, int n,

@@ -35,6 +35,7 @@
 #include "k_step3d.cuh"
 #include "pdl.cuh"
 #include "step2d_math.cuh"
+#include "taps.cuh"
 
 namespace fwi {
 namespace {
@@ -141,6 +142,11 @@ k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUte
             }
         }
     }
+    bool taps = false;   // an off-grid source's taps meet this thread's block
+    if (MODE != kImg && p.src_pts && left > 0) {
+        taps = taps_meet(p.src_pts[shot], 2, zr, RZ, 0, 1, x0);
+        if (taps) srcv = p.dt2 * p.wavelet[(int64_t)shot * p.nt + n];
+    }
     float sca = 1.0f, scd = 1.0f;
     char *codes = nullptr;
     if (MODE == kStore) {
@@ -183,6 +189,7 @@ k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUte
         lap_x<M>(w, ctr[r], p.c, za[r], zb[r], l0, l1);
         const float4 c = ctr[r];
         float4 o = update4(c, l0, l1, pv[r], Wv[r], sx4, sz[r], (MODE != kImg && r == src_r) ? src_e : -1, srcv);
+        if (MODE != kImg && taps && in) add_taps(p.src_pts[shot], 2, zr + r, 0, x0, srcv, sz[r], sx4, o);
         if (p.rec_map && zr + r == p.rec_z && xin) {
             const int4 ri = __ldg((const int4 *)(p.rec_map + (int64_t)shot * plane + x0));
             const int idx[4] = {ri.x, ri.y, ri.z, ri.w};

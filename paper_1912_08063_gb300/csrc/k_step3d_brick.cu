@@ -31,6 +31,7 @@
 
 #include "k_step3d.cuh"
 #include "pdl.cuh"
+#include "taps.cuh"
 
 namespace fwi {
 namespace {
@@ -232,6 +233,11 @@ k_step3d_brick(const __grid_constant__ Step3dParams p, const __grid_constant__ C
             srcv = p.dt2 * p.wavelet[(int64_t)shot * p.nt + n];
         }
     }
+    bool taps = false;   // an off-grid source's taps meet this thread's block
+    if (MODE != kModeAdj && p.src_pts) {
+        taps = taps_meet(p.src_pts[shot], 3, zb, RZ, y0, RY, x0);
+        if (taps) srcv = p.dt2 * p.wavelet[(int64_t)shot * p.nt + n];
+    }
     float sca = 1.0f, scd = 1.0f;
     if (MODE == kModeStepStore) {
         const float2 sc = store_scales(p.st_max, shot, p.st_dtype);
@@ -360,6 +366,12 @@ k_step3d_brick(const __grid_constant__ Step3dParams p, const __grid_constant__ C
             const float2 d1 = __fadd2_rn(make_float2(1.0f + sx.z, 1.0f + sx.w), make_float2(syz, syz));
             float2 o0 = __ffma2_rn(t0, make_float2(rcp_fast(d0.x), rcp_fast(d0.y)), lo2(A));
             float2 o1 = __ffma2_rn(t1, make_float2(rcp_fast(d1.x), rcp_fast(d1.y)), hi2(A));
+            if (MODE != kModeAdj && taps && ok[i][r]) {
+                float4 ov = make_float4(o0.x, o0.y, o1.x, o1.y);
+                add_taps(p.src_pts[shot], 3, z, y, x0, srcv, szr[i] + syr[r], sx, ov);
+                o0 = lo2(ov);
+                o1 = hi2(ov);
+            }
             if (p.rec_map && z == p.rec_z && ok[i][r]) {
                 float ov[4] = {o0.x, o0.y, o1.x, o1.y};
                 s3d::rec_epilogue<MODE>(p, shot, y, x0, n, ov);

@@ -42,6 +42,7 @@ struct Step3dParams {
     float *out;                   // the new state, over prev (in place)
     float *g;                     // kModeAdj: gradient accumulator
     const int64_t *src_off;       // may be null (kModeStep: injection; kModeAdj: g term)
+    const PointTaps *src_pts;     // brick kernel, forward modes: off-grid sources, or null
     const float *wavelet;
     int nt, n;
     const int *n_dev;             // nullable: the step index is *n_dev + n

@@ -818,19 +818,20 @@ int finish_output(void *user, const void *dev, size_t bytes, bool host, cudaStre
 
 namespace fwi {
 
-// CTAs per cluster with which a call on `ns` shots steps on chip, 0 if it does not: a 2-D
+// CTAs per cluster with which a call on `ns` shots steps on chip in `mode` (0 forward, 1 with
+// checkpoint stores, 2 reverse), 0 if it does not: a 2-D
 // grid whose states fit the shared memory of one cluster per shot, with node sources and
 // node receivers on one row, and no more shots than clusters run at once (a second wave
 // would double the time, while the tile kernel's launches take the same few microseconds
 // for a few small shots as for one).
-int onchip_size(fwi_model *m, int ns, bool reverse)
+int onchip_size(fwi_model *m, int ns, int mode)
 {
     if (m->ndim != 2 || m->opts.temporal_blocking == 1 || m->opts.timing || m->og_src || m->og_rec ||
         m->rec_fuse_z < 0)
         return 0;
     for (int i = 0; i < kOnchipSizes; ++i) {
         const int C = kOnchipSize[i];
-        if (!onchip2d_fits(m->g, C, reverse)) continue;
+        if (!onchip2d_fits(m->g, C, mode)) continue;
         if (m->cl_active[i] < 0) m->cl_active[i] = onchip2d_clusters(m->M, C);
         if (ns <= m->cl_active[i]) return C;
     }
@@ -842,6 +843,7 @@ Onchip2d onchip_params(const fwi_model *m, const StepParams &p, int ns, int C)
     Onchip2d a{};
     a.p = p;
     a.p.n_dev = nullptr;
+    a.p.err = m->d_flag;
     a.p.rec_map = m->rec_map.as<int>();
     a.p.rec_z = m->rec_fuse_z;
     a.p.nrec = m->geo_nrec;
@@ -916,7 +918,7 @@ int fwd_setup(FwdJob &j, fwi_model *m, int ns, int nr, const float *wav, float *
     j.uc = m->u[0].as<float>();
     j.up = m->u[1].as<float>();
     j.n = 0;
-    j.onchip = onchip_size(m, ns, false);
+    j.onchip = onchip_size(m, ns, 0);
     return FWI_OK;
 }
 
@@ -1353,8 +1355,8 @@ int grad_setup(GradJob &j, fwi_model *m, const fwi_acq *acq, const float *wavele
     // the step kernels compute the checkpoint max-abs when asked, unless off-grid source
     // taps are added after the step (then a separate max-abs pass sees the final state)
     j.fused_max = !m->og_src || j.pf.src_pts;
-    j.on_fwd = onchip_size(m, ns, false);
-    j.on_rev = onchip_size(m, ns, true);
+    j.on_fwd = onchip_size(m, ns, 1);
+    j.on_rev = onchip_size(m, ns, 2);
     if (j.on_fwd || j.on_rev) FWI_TRY(upload_onchip_schedule(m, s));
     return FWI_OK;
 }
@@ -1799,6 +1801,7 @@ int job_batch_entry(Job *j, Batch2dEntry *e, int zchunk)
     e->p.zchunk = zchunk;
     e->p.nzchunks = (m->g.nz + zchunk - 1) / zchunk;
     e->p.n_dev = nullptr;
+    e->p.err = f.m->d_flag;
     e->p.rec_tr = f.tr;
     e->p.rec_map = m->rec_fuse_z >= 0 ? m->rec_map.as<int>() : nullptr;
     e->p.rec_z = m->rec_fuse_z;

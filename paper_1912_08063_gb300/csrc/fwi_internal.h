@@ -163,8 +163,9 @@ cudaError_t launch_sample_multi(const Batch2d *tab, int t, int grid, cudaStream_
 constexpr int kOnchipSlot = (1 << 24) - 1;
 constexpr int kOnchipPairSlot = 1 << 24;   // the slot holds two fields per shot
 constexpr int kOnchipPair = 1 << 25;       // store the pair (u^n, u^n - u^{n-1}), not u^n alone
-// blocks of 4 x 2 points a thread may own (registers)
-constexpr int kOnchipFwdUnits = 4, kOnchipRevUnits = 2;
+// Blocks of 4 x 2 points a thread may own in mode 0 (forward), 1 (with checkpoint stores) and
+// 2 (reverse): as many as measured faster than single steps (k_step2d_onchip.cu).
+__host__ __device__ constexpr int onchip_units(int M, int mode) { return mode == 0 ? (M == 4 ? 4 : 2) : (M == 4 ? 2 : 1); }
 // CTAs per cluster, most first: the most that leave bands of M rows
 constexpr int kOnchipSizes = 3;
 constexpr int kOnchipSize[kOnchipSizes] = {16, 8, 4};
@@ -192,9 +193,9 @@ struct Onchip2d {
 // cluster2d_size: the cluster size to use (16, else 8; 0 if clusters cannot be launched).
 int cluster2d_size(int M);
 int cluster2d_max_smem();
-// whether grid g fits on C CTAs, the shared memory per CTA it takes, and the clusters that
+// whether grid g fits on C CTAs in a mode, the shared memory per CTA it takes, and the clusters that
 // run at once
-bool onchip2d_fits(const Geom &g, int C, bool reverse);
+bool onchip2d_fits(const Geom &g, int C, int mode);
 int onchip2d_smem(const Geom &g, int C);
 int onchip2d_clusters(int M, int C);
 // mode 0 forward, 1 forward with checkpoint stores, 2 reverse with imaging

@@ -6,21 +6,29 @@
 // either side, in two shared-memory buffers used alternately (u^n read, u^{n+1} written).  A
 // thread owns up to NU blocks of 4 columns x 2 rows for the whole launch and holds their W
 // and, in the reverse sweep, gradient sums in registers.  It writes new values
-// into its own CTA's next buffer and, near a band's edge, into the neighbour's halo rows
-// through distributed shared memory, so every read is local.  One cluster barrier per step
-// (hardware, nothing polls) orders both.  With checkpoints, the maxima that set a 16-bit
-// code's scale travel the same way: each CTA writes its own into every CTA's shared memory
-// before the barrier, and the next step, which stores the state, reduces them.
+// into its own CTA's next buffer and, near a band's edge, sends them into the neighbour's halo
+// rows (st.async, which counts its bytes on an mbarrier of the neighbour), so every read is
+// local.  A step waits for two things: a CTA barrier, and, for the threads whose rows read
+// halo rows, the neighbours' bytes.  That is enough: the threads that read a halo row are
+// those that send the rows next to it, so once a neighbour has a band's edge rows complete,
+// nobody reads the halo rows that it overwrites next.  With checkpoints, the maxima that set
+// a 16-bit code's scale travel the same way, each CTA's to every CTA; a step that stores the
+// state waits for them after its z-sums, and the first thread waits for them in every step,
+// so no CTA runs more than a step ahead of another there.
 //
-// Bound by latency: the barrier and the dependent shared-memory reads and sums of a step.
-// Measured on GB300 against single steps of the tile kernel (their launches bound them), us
-// per step, forward / gradient (a forward step with store and a reverse step, and the call's
-// fixed work), radius 4: 128^2 4.2 / 13.7 -> 1.2 / 4.8; 201^2 4.2 / 13.2 -> 1.5 / 5.8; 256^2
-// 4.2 / 14.9 -> 2.0 / 7.5; 384^2 4.2 / 15.8 -> 3.1 / 10.5 (computed grids of 168^2 to 424^2);
-// radius 8: 256^2 4.2 / 15.2 -> 2.8 / 8.9; four shots of 300^2 4.2 / 16.3 -> 2.3 / 9.3.
-// Clusters of 8 and of 4 CTAs are slower wherever 16 run (201^2: 2.4 and 4.1 forward), and
-// still beat single steps where they fit (128^2: 1.5 and 2.3), so they take the grids whose
-// bands 16 CTAs would cut below M rows and the calls with more shots than clusters of 16.
+// Bound by latency: the messages and the dependent shared-memory reads and sums of a step.
+// Measured on GB300 against single steps of the tile kernel (programmatic launches), us per
+// step, forward / gradient (a forward step with store and a reverse step, and the call's fixed
+// work), radius 4: 128^2 2.64 / 6.43 -> 1.00 / 3.74; 201^2 2.69 / 6.53 -> 1.28 / 4.64; 256^2
+// 2.74 / 6.61 -> 1.75 / 5.70; 384^2 forward 3.44 -> 3.06, 440^2 3.58 -> 3.55 (computed grids of
+// 168^2 to 480^2); radius 8: 256^2 forward 2.95 -> 2.41; four shots of 300^2 radius 4 3.56 /
+// 9.19 -> 2.04 / 6.86, eight of 201^2 on clusters of 8 3.67 / 9.20 -> 2.20 / 7.14.  Not taken,
+// since no faster: gradients with three blocks a thread at radius 4 (320^2 7.77 -> 7.95) or two
+// at radius 8 (256^2 7.40 -> 7.57), forward steps with three at radius 8 (384^2 3.99 -> 4.21).
+// With a cluster barrier per step instead of the messages: 201^2 1.52 / 5.75, 256^2 1.97 /
+// 7.47.  Clusters of 8 and of 4 CTAs are slower wherever 16 run (201^2 forward 2.4 and 4.1 with
+// the barrier) and still beat single steps where they fit, so they take the grids whose bands
+// 16 CTAs would cut below M rows and the calls with more shots than clusters of 16.
 #include <cooperative_groups.h>
 
 #include "code16.cuh"
@@ -38,6 +46,9 @@ using s2d::lo2;
 using s2d::update4;
 using s2d::z_block;
 using s3d::absmax_nan;
+using s3d::mbar_expect_tx;
+using s3d::mbar_init;
+using s3d::smem_u32;
 
 constexpr int kT = 512;        // threads per CTA
 constexpr int kRZ = 2;         // rows per block
@@ -68,6 +79,45 @@ __device__ __forceinline__ char *slot_codes(const OnchipCkpt &a, int64_t field, 
     return a.codes + __ldg(a.slot_off + (d & kOnchipSlot)) * a.half_slot + (int64_t)shot * cs * (a.dtype == 0 ? 4 : 2);
 }
 
+// Bounded wait (about 2^22 polls) for a phase that other CTAs of the cluster complete.
+__device__ __forceinline__ bool wait_cluster(uint64_t *bar, uint32_t parity)
+{
+    for (int i = 0; i < (1 << 22); ++i) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+
+__device__ __forceinline__ uint32_t in_cta(const void *p, int rank)   // p in CTA `rank` of the cluster
+{
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    return r;
+}
+
+// Sends 16 or 8 bytes to another CTA's shared memory and counts them on its barrier `bar`.
+__device__ __forceinline__ void send(uint32_t addr, float4 v, uint32_t bar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar)
+                 : "memory");
+}
+
+__device__ __forceinline__ void send(uint32_t addr, uint2 v, uint32_t bar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.u32 [%0], {%1, %2}, [%3];"
+                 ::"r"(addr), "r"(v.x), "r"(v.y), "r"(bar)
+                 : "memory");
+}
+
 template <int M, int MODE, int NU>
 __device__ __forceinline__ void advance(const OnchipCkpt &a, const StepParams &p, float *u0, float *u1,
                                         int n0, int k, float *smem, int shot)
@@ -82,7 +132,24 @@ __device__ __forceinline__ void advance(const OnchipCkpt &a, const StepParams &p
     float *buf0 = smem, *buf1 = smem + l.rows * SX;
     float *sxs = smem + 2 * l.rows * SX, *szs = sxs + 4 * G;
     __shared__ uint2 cmax[2][kMaxC];    // per parity, each CTA's maxima of the new state
-    __shared__ uint2 wmax[kT / 32];
+    __shared__ uint2 wmax[2][kT / 32];
+    // arrivals of state t: halo rows on halo_bar[t & 1], maxima on max_bar[t & 1]
+    __shared__ __align__(8) uint64_t halo_bar[2], max_bar[2];
+    bool dead = false;                  // a bounded wait of this thread gave up: it waits no more
+    auto wait_for = [&](uint64_t *bar, int use) {
+        if (dead || wait_cluster(bar, use & 1)) return;
+        dead = true;
+        atomicOr(p.err, 2u);
+    };
+    if (tid == 0) {
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(halo_bar + i, 1);
+            mbar_init(max_bar + i, 1);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        if (MODE == kCkpt) mbar_expect_tx(max_bar, 8 * C);   // state 0
+    }
+    const uint32_t halo_bytes = (uint32_t)((rank > 0) + (rank < C - 1)) * M * G * 16;
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
 
     for (int i = tid; i < l.rows * SX / 2; i += kT) ((float4 *)smem)[i] = zero4;   // both buffers
@@ -102,6 +169,7 @@ __device__ __forceinline__ void advance(const OnchipCkpt &a, const StepParams &p
     int soff[NU], goff[NU], lr0[NU];    // shared offset of the z-walk's first row, field offset
     float4 Wv[NU][kRZ], gv[MODE == kRev ? NU : 1][kRZ];
     uint4 ur[MODE == kRev ? NU : 1][kRZ];
+    bool edge = false;                  // some of them read halo rows
     int src_u = -1, src_r = 0, src_e = 0, rec_u = -1, rec_r = 0;
     int4 ri = make_int4(-1, -1, -1, -1);
     const int64_t so = p.src_off ? p.src_off[shot] : -1;
@@ -112,6 +180,7 @@ __device__ __forceinline__ void advance(const OnchipCkpt &a, const StepParams &p
         const int g = id % G;
         soff[u] = lr0[u] * SX + M + 4 * g;
         goff[u] = (r0 + lr0[u]) * px + 4 * g;
+        edge |= lr0[u] < R && (lr0[u] < M || lr0[u] + kRZ > R - M);
 #pragma unroll
         for (int r = 0; r < kRZ; ++r) {
             const bool in = lr0[u] + r < R;
@@ -130,34 +199,48 @@ __device__ __forceinline__ void advance(const OnchipCkpt &a, const StepParams &p
             }
         }
     }
-    // The maxima of the newest state over the cluster, into cmax[par] of every CTA (complete
-    // after the next cluster barrier).
-    auto share_max = [&](float mxa, float mxd, int par) {
-        const unsigned wa = __reduce_max_sync(0xffffffffu, __float_as_uint(mxa) & 0x7fffffffu);
-        const unsigned wd = __reduce_max_sync(0xffffffffu, __float_as_uint(mxd) & 0x7fffffffu);
-        if ((tid & 31) == 0) wmax[tid >> 5] = make_uint2(wa, wd);
+    // The end of a step that made state t: a CTA barrier and, with checkpoints, this CTA's
+    // maxima of the state into cmax[t & 1] of every CTA.
+    auto end_step = [&](float mxa, float mxd, int t) {
+        if (MODE == kCkpt) {
+            const unsigned wa = __reduce_max_sync(0xffffffffu, __float_as_uint(mxa) & 0x7fffffffu);
+            const unsigned wd = __reduce_max_sync(0xffffffffu, __float_as_uint(mxd) & 0x7fffffffu);
+            if ((tid & 31) == 0) wmax[t & 1][tid >> 5] = make_uint2(wa, wd);
+        }
         __syncthreads();
-        if (tid < 32) {
-            const uint2 w = tid < kT / 32 ? wmax[tid] : make_uint2(0u, 0u);
+        if (MODE == kCkpt && tid < 32) {
+            const uint2 w = tid < kT / 32 ? wmax[t & 1][tid] : make_uint2(0u, 0u);
             const uint2 c = make_uint2(__reduce_max_sync(0xffffffffu, w.x), __reduce_max_sync(0xffffffffu, w.y));
-            if (tid < C) *cl.map_shared_rank(&cmax[par][rank], tid) = c;
+            if (tid < C) send(in_cta(&cmax[t & 1][rank], tid), c, in_cta(max_bar + (t & 1), tid));
         }
     };
-    auto state_max = [&](int par) {
+    // The maxima of state t over the cluster, once they have arrived.
+    auto state_max = [&](int t) {
+        wait_for(max_bar + (t & 1), t >> 1);
+        __syncwarp();
         const int i = tid & 31;
-        const uint2 c = i < C ? cmax[par][i] : make_uint2(0u, 0u);
+        const uint2 c = i < C ? cmax[t & 1][i] : make_uint2(0u, 0u);
         return make_uint2(__reduce_max_sync(0xffffffffu, c.x), __reduce_max_sync(0xffffffffu, c.y));
     };
     // operands of step s that come from global memory, one step ahead
     float srcv = 0.0f, ainv = 1.0f;
     float4 inj = zero4;
+    // the schedule entry of the next step to fetch and its codes, found one step earlier still
+    int nd = -1;
+    char *ncodes = nullptr;
+    auto look_up = [&](int s) {
+        if (MODE == kFwd || s >= k) return;
+        nd = __ldg(a.desc + s);
+        if (nd >= 0) ncodes = slot_codes(a, p.g.field, nd, shot);
+    };
     auto fetch = [&](int s) {
         if (s >= k) return;
         const int n = MODE == kRev ? n0 - s : n0 + s;
         if (src_u >= 0) srcv = p.dt2 * p.wavelet[(int64_t)shot * p.nt + n];
         if (MODE == kRev) {
-            const int d = __ldg(a.desc + s);
-            const char *codes = slot_codes(a, p.g.field, d, shot);
+            const int d = nd;
+            const char *codes = ncodes;
+            look_up(s + 1);
             ainv = a.dtype == 0 ? 1.0f : 1.0f / a.scales[((int64_t)(d & kOnchipSlot) * a.ns + shot) * 2];
 #pragma unroll
             for (int u = 0; u < NU; ++u)
@@ -190,6 +273,7 @@ __device__ __forceinline__ void advance(const OnchipCkpt &a, const StepParams &p
 #pragma unroll
             for (int r = 0; r < kRZ; ++r) ur[u][r] = make_uint4(0u, 0u, 0u, 0u);
     }
+    look_up(0);
     fetch(0);
     if (MODE == kCkpt) {
         __syncthreads();   // the states are loaded
@@ -206,42 +290,56 @@ __device__ __forceinline__ void advance(const OnchipCkpt &a, const StepParams &p
                     mxd = absmax_nan(absmax_nan(absmax_nan(absmax_nan(mxd, c.x - v.x), c.y - v.y), c.z - v.z), c.w - v.w);
                 }
         }
-        cl.sync();         // every CTA runs: its shared memory may be written
-        share_max(mxa, mxd, 0);
+        cl.sync();         // every CTA runs and its barriers are initialised
+        end_step(mxa, mxd, 0);
+    } else {
+        cl.sync();
     }
-    cl.sync();
+    // the neighbours' copies of this CTA's edge rows, as offsets to a row's place in a buffer
+    const uint32_t up_s = rank > 0 ? in_cta(smem, rank - 1) + (Rup + M) * SX * 4 : 0u;
+    const uint32_t up_b = rank > 0 ? in_cta(halo_bar, rank - 1) : 0u;
+    const uint32_t dn_s = rank < C - 1 ? in_cta(smem, rank + 1) - (R - M) * SX * 4 : 0u;
+    const uint32_t dn_b = rank < C - 1 ? in_cta(halo_bar, rank + 1) : 0u;
 
     for (int s = 0; s < k; ++s) {
         const int n = MODE == kRev ? n0 - s : n0 + s;
         float *cur = (s & 1) ? buf1 : buf0, *nxt = (s & 1) ? buf0 : buf1;
-        float *up = rank > 0 ? cl.map_shared_rank(nxt, rank - 1) + (Rup + M) * SX : nullptr;
-        float *dn = rank < C - 1 ? cl.map_shared_rank(nxt, rank + 1) - (R - M) * SX : nullptr;
-        int st = -1;
+        const int par = (s + 1) & 1;                       // of the state this step makes
+        const uint32_t nxt_off = par ? l.rows * SX * 4 : 0;
+        // state s's halo rows, and the counts of the messages this step's neighbours send
+        if (s > 0 && (tid == 0 || edge)) wait_for(halo_bar + (s & 1), (s - 1) >> 1);
+        if (tid == 0 && !dead) {
+            mbar_expect_tx(halo_bar + par, halo_bytes);
+            if (MODE == kCkpt) mbar_expect_tx(max_bar + par, 8 * C);
+        }
+        const int st = MODE == kCkpt && (s > 0 || a.first_store) ? nd : -1;
+        char *codes = ncodes;
         float sca = 1.0f, scd = 1.0f;
-        char *codes = nullptr;
-        if (MODE == kCkpt && (s > 0 || a.first_store)) {
-            st = __ldg(a.desc + s);
+        float mxa = 0.0f, mxd = 0.0f;
+        float2 za[kRZ], zb[kRZ];
+        float4 ctr[kRZ];
+        if (lr0[0] < R) z_block<M, kRZ>(cur + soff[0], SX, p.c, ctr, za, zb);
+        if (MODE == kCkpt) {
+            look_up(s + 1);
             if (st >= 0) {
-                const uint2 m = state_max(s & 1);
+                const uint2 m = state_max(s);
                 sca = snap_scale(m.x, a.dtype);
                 scd = snap_scale(m.y, a.dtype);
-                codes = slot_codes(a, p.g.field, st, shot);
                 if (rank == 0 && tid == 0) {
                     float *sc = a.scales + ((int64_t)(st & kOnchipSlot) * a.ns + shot) * 2;
                     sc[0] = sca;
                     sc[1] = scd;
                     if (m.x >= 0x7f800000u) atomicOr(a.flag, 1u);
                 }
+            } else if (tid == 0) {
+                wait_for(max_bar + (s & 1), s >> 1);
             }
         }
-        float mxa = 0.0f, mxd = 0.0f;
 #pragma unroll
         for (int u = 0; u < NU; ++u) {
             if (lr0[u] >= R) continue;
             const float *col = cur + soff[u];
-            float2 za[kRZ], zb[kRZ];
-            float4 ctr[kRZ];
-            z_block<M, kRZ>(col, SX, p.c, ctr, za, zb);
+            if (u > 0) z_block<M, kRZ>(col, SX, p.c, ctr, za, zb);
             const int xg = (soff[u] - lr0[u] * SX - M);   // first column of the group
             const float4 sx = *(const float4 *)(sxs + xg);
 #pragma unroll
@@ -280,8 +378,9 @@ __device__ __forceinline__ void advance(const OnchipCkpt &a, const StepParams &p
                 }
                 const int x = M + xg;
                 *(float4 *)own = o;
-                if (lr < M && rank > 0) *(float4 *)(up + lr * SX + x) = o;
-                if (lr >= R - M && rank < C - 1) *(float4 *)(dn + lr * SX + x) = o;
+                const uint32_t to = nxt_off + (uint32_t)(lr * SX + x) * 4;
+                if (lr < M && rank > 0) send(up_s + to, o, up_b + 8 * par);
+                if (lr >= R - M && rank < C - 1) send(dn_s + to, o, dn_b + 8 * par);
                 if (MODE == kCkpt) {
                     mxa = absmax_nan(absmax_nan(absmax_nan(absmax_nan(mxa, o.x), o.y), o.z), o.w);
                     mxd = absmax_nan(absmax_nan(absmax_nan(absmax_nan(mxd, o.x - c.x), o.y - c.y), o.z - c.z), o.w - c.w);
@@ -313,10 +412,14 @@ __device__ __forceinline__ void advance(const OnchipCkpt &a, const StepParams &p
             }
         }
         fetch(s + 1);
-        if (MODE == kCkpt) share_max(mxa, mxd, (s + 1) & 1);
-        // every band's new state, halo rows and maxima are written, every read is done
-        cl.sync();
+        end_step(mxa, mxd, s + 1);
     }
+    // no message may be on its way to a CTA that ends
+    if (tid == 0) {
+        wait_for(halo_bar + (k & 1), (k - 1) >> 1);
+        if (MODE == kCkpt) wait_for(max_bar + (k & 1), k >> 1);
+    }
+    cl.sync();
     // back to global memory, in the buffers that k single steps would leave
     float *newest = (k & 1) ? u1 : u0, *older = (k & 1) ? u0 : u1;
     const float *cur = (k & 1) ? buf1 : buf0, *old = (k & 1) ? buf0 : buf1;
@@ -331,7 +434,7 @@ __device__ __forceinline__ void advance(const OnchipCkpt &a, const StepParams &p
             if (MODE == kRev) *(float4 *)(p.gacc + (int64_t)shot * p.g.field + o) = gv[u][r];
         }
     if (MODE == kCkpt) {
-        const uint2 m = state_max(k & 1);
+        const uint2 m = state_max(k);
         if (rank == 0 && tid == 0) {
             a.maxbits[2 * shot] = m.x;
             a.maxbits[2 * shot + 1] = m.y;
@@ -359,7 +462,7 @@ __global__ void __launch_bounds__(kT, 1) k_step2d_cluster(const Batch2d *__restr
     const Batch2dEntry &E = tab->e[req];
     const OnchipCkpt none{};
     const int left = E.p.nt - E.n0;
-    if (left > 0) advance<M, kFwd, kOnchipFwdUnits>(none, E.p, E.u0, E.u1, E.n0, left < k ? left : k, smem, 0);
+    if (left > 0) advance<M, kFwd, onchip_units(M, kFwd)>(none, E.p, E.u0, E.u1, E.n0, left < k ? left : k, smem, 0);
 }
 
 typedef void (*OnchipKernel)(const Onchip2d);
@@ -367,12 +470,14 @@ typedef void (*OnchipKernel)(const Onchip2d);
 template <int M, int MODE>
 OnchipKernel onchip_kernel(int nu)
 {
+    constexpr int most = onchip_units(M, MODE);
     if (nu == 1) return k_step2d_onchip<M, MODE, 1>;
-    if (nu == 2) return k_step2d_onchip<M, MODE, 2>;
-    if constexpr (MODE != kRev) {
+    if constexpr (most >= 2)
+        if (nu == 2) return k_step2d_onchip<M, MODE, 2>;
+    if constexpr (most >= 3)
         if (nu == 3) return k_step2d_onchip<M, MODE, 3>;
+    if constexpr (most >= 4)
         if (nu == 4) return k_step2d_onchip<M, MODE, 4>;
-    }
     return nullptr;
 }
 
@@ -444,12 +549,12 @@ int onchip2d_smem(const Geom &g, int C)
     return (layout_of(g.nz, g.nx, g.M, C).floats * 4 + 1023) / 1024 * 1024;
 }
 
-bool onchip2d_fits(const Geom &g, int C, bool reverse)
+bool onchip2d_fits(const Geom &g, int C, int mode)
 {
     // bands of at least M rows (halos reach the next CTA only), no more than one row of
     // blocks per pass over the threads (a thread then meets the receiver row once)
     return C > 0 && g.ndim == 2 && g.nz / C >= g.M && (g.nx + 3) / 4 <= kT &&
-           units_of(g, C) <= (reverse ? kOnchipRevUnits : kOnchipFwdUnits) && onchip2d_smem(g, C) <= kSmemMax;
+           units_of(g, C) <= onchip_units(g.M, mode) && onchip2d_smem(g, C) <= kSmemMax;
 }
 
 int cluster2d_size(int M)

@@ -332,7 +332,7 @@ extern "C" int fwi_serve(const fwi_request *reqs, int32_t n, const fwi_serve_opt
                 int kind = 0;
                 const int C = cl_size[ri];
                 if (C > 0 && fwi::job_batch_entry(free_slot->job, &probe, 64) == FWI_OK &&
-                    probe.p.rec_map && fwi::onchip2d_fits(probe.p.g, C, false))
+                    probe.p.rec_map && fwi::onchip2d_fits(probe.p.g, C, 0))
                     kind = 1;
                 const int pi = (kind * 2 + ri) * kPools + (rr++ % kPools);
                 Pool &pl = pools[pi];

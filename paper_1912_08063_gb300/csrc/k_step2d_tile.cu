@@ -68,7 +68,9 @@ __device__ __forceinline__ void tma_tile(void *dst, const CUtensorMap *map, int 
 constexpr int kWarps = 2, kMinCtas = 8;
 __host__ __device__ constexpr int tile_rz(int mode) { return mode == kImg ? 3 : 4; }
 
-template <int M, int MODE>
+// TAPS: an off-grid source is added too (an instantiation of its own, so that the common one
+// pays nothing for it: 3 % of a 64-shot step).
+template <int M, int MODE, bool TAPS>
 __global__ void __launch_bounds__(32 * kWarps, kMinCtas)
 k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUtensorMap map)
 {
@@ -143,7 +145,7 @@ k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUte
         }
     }
     bool taps = false;   // an off-grid source's taps meet this thread's block
-    if (MODE != kImg && p.src_pts && left > 0) {
+    if (TAPS && left > 0) {
         taps = taps_meet(p.src_pts[shot], 2, zr, RZ, 0, 1, x0);
         if (taps) srcv = p.dt2 * p.wavelet[(int64_t)shot * p.nt + n];
     }
@@ -189,7 +191,7 @@ k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUte
         lap_x<M>(w, ctr[r], p.c, za[r], zb[r], l0, l1);
         const float4 c = ctr[r];
         float4 o = update4(c, l0, l1, pv[r], Wv[r], sx4, sz[r], (MODE != kImg && r == src_r) ? src_e : -1, srcv);
-        if (MODE != kImg && taps && in) add_taps(p.src_pts[shot], 2, zr + r, 0, x0, srcv, sz[r], sx4, o);
+        if (TAPS && taps && in) add_taps(p.src_pts[shot], 2, zr + r, 0, x0, srcv, sz[r], sx4, o);
         if (p.rec_map && zr + r == p.rec_z && xin) {
             const int4 ri = __ldg((const int4 *)(p.rec_map + (int64_t)shot * plane + x0));
             const int idx[4] = {ri.x, ri.y, ri.z, ri.w};
@@ -253,7 +255,9 @@ cudaError_t go(const StepParams &p, int nshots, const CUtensorMap &map, cudaStre
 {
     constexpr int TZ = kWarps * tile_rz(MODE);
     const dim3 grid((p.g.nx + kTileX - 1) / kTileX, (p.g.nz + TZ - 1) / TZ, nshots);
-    return launch_pdl(k_step2d_tile<M, MODE>, grid, dim3(32 * kWarps), 0, s, p, map);
+    if (MODE != kImg && p.src_pts)
+        return launch_pdl(k_step2d_tile<M, MODE, MODE != kImg>, grid, dim3(32 * kWarps), 0, s, p, map);
+    return launch_pdl(k_step2d_tile<M, MODE, false>, grid, dim3(32 * kWarps), 0, s, p, map);
 }
 
 }  // namespace

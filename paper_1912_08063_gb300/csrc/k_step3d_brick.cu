@@ -148,7 +148,8 @@ __device__ __forceinline__ void plane_xy(const Step3dParams &p, const float *hk,
     }
 }
 
-template <int M, int MODE, bool ISO>
+// TAPS: an off-grid source is added too (an instantiation of its own).
+template <int M, int MODE, bool ISO, bool TAPS>
 __global__ void __launch_bounds__(Brick<M, MODE, ISO>::NT, Brick<M, MODE, ISO>::MINB)
 k_step3d_brick(const __grid_constant__ Step3dParams p, const __grid_constant__ CUtensorMap map_mid,
                const __grid_constant__ CUtensorMap map_arm, int tiles_z)
@@ -234,7 +235,7 @@ k_step3d_brick(const __grid_constant__ Step3dParams p, const __grid_constant__ C
         }
     }
     bool taps = false;   // an off-grid source's taps meet this thread's block
-    if (MODE != kModeAdj && p.src_pts) {
+    if (TAPS) {
         taps = taps_meet(p.src_pts[shot], 3, zb, RZ, y0, RY, x0);
         if (taps) srcv = p.dt2 * p.wavelet[(int64_t)shot * p.nt + n];
     }
@@ -366,7 +367,7 @@ k_step3d_brick(const __grid_constant__ Step3dParams p, const __grid_constant__ C
             const float2 d1 = __fadd2_rn(make_float2(1.0f + sx.z, 1.0f + sx.w), make_float2(syz, syz));
             float2 o0 = __ffma2_rn(t0, make_float2(rcp_fast(d0.x), rcp_fast(d0.y)), lo2(A));
             float2 o1 = __ffma2_rn(t1, make_float2(rcp_fast(d1.x), rcp_fast(d1.y)), hi2(A));
-            if (MODE != kModeAdj && taps && ok[i][r]) {
+            if (TAPS && taps && ok[i][r]) {
                 float4 ov = make_float4(o0.x, o0.y, o1.x, o1.y);
                 add_taps(p.src_pts[shot], 3, z, y, x0, srcv, szr[i] + syr[r], sx, ov);
                 o0 = lo2(ov);
@@ -426,7 +427,8 @@ template <int M, int MODE, bool ISO>
 cudaError_t go(const Step3dParams &p, int nshots, const CUtensorMap &mid, const CUtensorMap &arm, cudaStream_t s)
 {
     using C = Brick<M, MODE, ISO>;
-    auto fn = k_step3d_brick<M, MODE, ISO>;
+    auto fn = MODE != kModeAdj && p.src_pts ? k_step3d_brick<M, MODE, ISO, MODE != kModeAdj>
+                                            : k_step3d_brick<M, MODE, ISO, false>;
     cudaError_t e = cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute((const void *)fn, cudaFuncAttributePreferredSharedMemoryCarveout,

@@ -203,8 +203,8 @@ int fwi_misfit_noalloc(const float *d_mod, const float *d_obs, int64_t n, double
  * s = 2^floor(log2(T / max|component|)), T = 2^14 for FP16 and 1 for BF16 (s = 1 for an
  * all-zero component): code holds [2][n] 16-bit values, scale[0..1] receive (s_a, s_d).
  * FWI_SNAP_FP32 copies a and b ([2][n] FP32, scales 1).  Non-finite input sets the
- * scales to NaN and returns FWI_OK (the codes are then unspecified).  Allocates two
- * words of stream-ordered scratch. */
+ * scales to NaN and returns FWI_OK (the codes are then unspecified).  Allocates nothing
+ * (scale holds the maxima until the scales replace them). */
 int fwi_snapshot_encode(const float *a, const float *b, int64_t n, int32_t dtype,
                         void *code, float *scale, cudaStream_t stream);
 /* Inverse of fwi_snapshot_encode: a = code[0] / s_a, b = a - code[1] / s_d. */

@@ -1511,14 +1511,18 @@ int grad_advance(GradJob &j, int64_t units, bool *done)
                 ++j.ia;
                 continue;
             }
-            if (!have_max) {
+            // FP32 stores need no maxima (the encode pass looks for non-finite values itself)
+            const bool fp32 = m->opts.snap_dtype == FWI_SNAP_FP32;
+            if (!have_max && !fp32) {
                 FWI_CU(cudaMemsetAsync(m->maxbits.p, 0, 2 * ns * sizeof(unsigned), s));
                 FWI_LAUNCH(m, launch_maxabs(m->u[j.cur].as<float>(), m->u[1 - j.cur].as<float>(),
                                             g.field, g.field, ns, m->maxbits.as<unsigned>(), s));
             }
             FWI_LAUNCH(m, launch_encode(m->u[j.cur].as<float>(), m->u[1 - j.cur].as<float>(),
                                         g.field, g.field, ns, m->opts.snap_dtype,
-                                        have_max ? j.ring_at(j.ring) : m->maxbits.as<unsigned>(),
+                                        fp32 && !have_max ? nullptr
+                                        : have_max        ? j.ring_at(j.ring)
+                                                          : m->maxbits.as<unsigned>(),
                                         (void *)(j.codes + m->slot_off[arg] * j.half_slot), slot_cstride(m, arg),
                                         m->scales.as<float>() + (size_t)arg * 2 * ns, m->d_flag,
                                         comps, s));
@@ -2126,14 +2130,7 @@ int fwi_snapshot_encode(const float *a, const float *b, int64_t n, int32_t dtype
 {
     if (!a || !b || !code || !scale || n < 0 || dtype < 0 || dtype > 2)
         return fail(FWI_ERR_ARG, "bad argument");
-    unsigned *mb = nullptr;
-    FWI_CU(cudaMallocAsync((void **)&mb, 2 * sizeof(unsigned), s));
-    FWI_CU(cudaMemsetAsync(mb, 0, 2 * sizeof(unsigned), s));
-    cudaError_t e = launch_maxabs(a, b, n, n, 1, mb, s);
-    if (e == cudaSuccess) e = launch_encode(a, b, n, n, 1, dtype, mb, code, 2 * n, scale, nullptr, 2, s);
-    cudaError_t e2 = cudaFreeAsync(mb, s);
-    if (e != cudaSuccess || e2 != cudaSuccess)
-        return fail(FWI_ERR_CUDA, std::string("encode: ") + cudaGetErrorString(e != cudaSuccess ? e : e2));
+    FWI_CU(launch_encode_pair(a, b, n, dtype, code, scale, s));
     return FWI_OK;
 }
 

@@ -242,11 +242,16 @@ cudaError_t launch_misfit(const float *d, const float *dobs, float *r_out, int64
 int misfit_blocks(int64_t n);
 cudaError_t launch_maxabs(const float *a, const float *b, int64_t n, int64_t stride,
                           int nshots, unsigned *maxbits, cudaStream_t s);
-// comps = 2: the pair (a, b); comps = 1: a only (a checkpoint restored only for imaging)
+// comps = 2: the pair (a, b); comps = 1: a only (a checkpoint restored only for imaging).
+// maxbits null: the scales are read from scale (16-bit), or 1 and non-finite values raise
+// flag (FP32)
 cudaError_t launch_encode(const float *a, const float *b, int64_t n, int64_t stride,
                           int nshots, int dtype, const unsigned *maxbits, void *code,
                           int64_t code_stride, float *scale, unsigned *flag, int comps,
                           cudaStream_t s);
+// the codec's encode of one pair: maxima, scales and codes, without scratch memory
+cudaError_t launch_encode_pair(const float *a, const float *b, int64_t n, int dtype, void *code,
+                               float *scale, cudaStream_t s);
 cudaError_t launch_decode(const void *code, int64_t code_stride, const float *scale,
                           int64_t n, int64_t stride, int nshots, int dtype, float *a, float *b,
                           int comps, cudaStream_t s);

@@ -1781,6 +1781,9 @@ bool job_batchable(const Job *j)
     return m->ndim == 2 && j->f.ns == 1 && !m->og_src && !m->og_rec && !m->opts.timing && j->f.tr != nullptr;
 }
 
+// Whether the job's turns are runs of steps on chip.
+bool job_onchip(const Job *j) { return j->kind == 0 ? j->f.onchip > 0 : j->gj.on_fwd > 0; }
+
 int job_batch_entry(Job *j, Batch2dEntry *e, int zchunk)
 {
     if (!job_batchable(j)) return fail(FWI_ERR_ARG, "job not eligible for the shared launch");

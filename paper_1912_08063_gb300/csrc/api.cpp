@@ -682,9 +682,7 @@ int step3d_launch(fwi_model *m, const StepParams &p, int ns, int mode, cudaStrea
         FWI_TRY(field_map(m, p.gacc, ns, 64, TY, &me));
     }
     const int tiles = ((g.nx + 63) / 64) * ((g.ny + TY - 1) / TY);
-    // z-parts in step when the streamed field is larger than the L2 (~126 MB)
-    const bool in_step = (double)g.field * 4.0 * ns > 96.0 * (1 << 20);
-    const int ctas = plan_persistent(q, tiles * ns, m->resident[mode], in_step);
+    const int ctas = plan_persistent(q, tiles * ns, m->resident[mode], true);
     FWI_CU(launch_step3d_tma(q, mode, ctas, mc, ma, mb, md, me, s));
     return FWI_OK;
 }

@@ -458,10 +458,10 @@ void brick_boxes(int M, int (&mid)[3], int (&arm)[3])
 }
 
 // Whether a launch takes bricks: up to the points of all shots below which they measured
-// faster than streaming (radius 4: forward modes equal at 200^3 computed points and 1.5x
-// faster at 168^3, reverse 0.9x at 168^3 and 1.35x at 136^3; radius 8: 1.2 to 1.3x at 200^3
-// and 0.9 to 0.95x at 232^3).  FWI_STEP3D_BRICK=0/1 overrides; the switches that choose
-// among the streaming kernels turn bricks off.
+// faster than streaming.  Radius 4: forward 0.85x at 200^3 computed points, 1.1x at 192^3 and
+// 1.4x at 176^3, reverse 0.9x at 176^3 and 1.35x at 136^3.  Radius 8: 1.2 to 1.3x at 200^3, 1.03
+// to 1.13x at 224^3, 0.86 to 1.0x at 232^3.  FWI_STEP3D_BRICK=0/1 overrides; the switches that
+// choose among the streaming kernels turn bricks off.
 bool step3d_use_brick(const Step3dParams &p, int mode)
 {
     if (const char *e = std::getenv("FWI_STEP3D_BRICK")) return std::atoi(e) != 0;
@@ -469,7 +469,7 @@ bool step3d_use_brick(const Step3dParams &p, int mode)
         if (std::getenv(v)) return false;
     const double points = (double)p.nx * p.ny * p.nz * p.nshots;
     if (p.M == 4) return points <= (mode == kModeAdj ? 3.5e6 : 7.5e6);
-    return points <= 10.0e6;
+    return points <= 11.5e6;
 }
 
 cudaError_t launch_step3d_brick(const Step3dParams &p, int mode, const CUtensorMap &mid,

@@ -108,6 +108,28 @@ __global__ void k_inject_pts(Geom g, float *__restrict__ f, const PointTaps *__r
     }
 }
 
+// Adds a row of taps at p, whose first column is `lead` columns past a group of four, as one
+// 16-byte addition per group it meets (three; rows are 32-byte aligned, so a group lies in its
+// row).  Columns of a group outside the taps receive a zero.  What bounds k_adjoint_pts is the
+// rate of its atomic additions: 16384 receivers on 256^3 took 104 us with one per tap; with one
+// per group the gradient call went from 204.7 to 187.7 ms, on 96^3 at 16th order from 35.7 to 32.0.
+__device__ __forceinline__ void add_row(float *p, int lead, const float (&v)[kTaps])
+{
+    float4 *b = (float4 *)(p - lead);
+    float e[kTaps + 4];
+#pragma unroll
+    for (int c = 0; c < kTaps + 4; ++c) e[c] = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (lead == k) {
+#pragma unroll
+            for (int c = 0; c < kTaps; ++c) e[k + c] = v[c];
+        }
+    atomicAdd(b, make_float4(e[0], e[1], e[2], e[3]));
+    atomicAdd(b + 1, make_float4(e[4], e[5], e[6], e[7]));
+    if (lead) atomicAdd(b + 2, make_float4(e[8], e[9], e[10], e[11]));
+}
+
 // The point work of reverse step m, one thread per row of taps:
 //   receivers (npts of them): the image term g += 2 wt u^m r[s][m-1][r] (u^m = x, FP32 or a
 //   code) and the injection mu^m += factor (W / a+) wt r, whose weights they share;
@@ -133,6 +155,7 @@ __global__ void k_adjoint_pts(Geom g, AdjointPts a)
         const float inv = (a.xfmt != 0 && a.xscale) ? 1.0f / a.xscale[2 * s] : 1.0f;
         const float syz = a.sz[t.z] + (g.ndim == 3 ? a.sy[t.y] : 0.0f);
         float *fs = a.mu + (int64_t)s * g.field, *gs = a.g + (int64_t)s * g.field;
+        float gv[kTaps], fv[kTaps];
 #pragma unroll
         for (int c = 0; c < kTaps; ++c) {
             const int64_t o = t.off + c;
@@ -140,10 +163,12 @@ __global__ void k_adjoint_pts(Geom g, AdjointPts a)
             float xv;
             if (a.xfmt == 0) xv = ((const float *)a.x)[(int64_t)s * a.xstride + o];
             else xv = code16_to_float(((const unsigned short *)a.x)[(int64_t)s * a.xstride + o], a.xfmt) * inv;
-            atomicAdd(gs + o, 2.0f * q * t.wzy * w * xv);
+            gv[c] = 2.0f * q * t.wzy * w * xv;
             const float ap = 1.0f + syz + a.sx[t.x0 + c];
-            atomicAdd(fs + o, q * t.wzy * w * (a.factor * a.W[o] / ap));
+            fv[c] = q * t.wzy * w * (a.factor * a.W[o] / ap);
         }
+        add_row(gs + t.off, t.x0 & 3, gv);
+        add_row(fs + t.off, t.x0 & 3, fv);
     } else {
         const float val = -a.dt2 * a.wav[(int64_t)pi * a.nt + a.m];
         const float *ms = a.mu1 + (int64_t)pi * g.field;
@@ -180,6 +205,20 @@ __global__ void k_gather_src_pts(Geom g, const float *__restrict__ f,
 
 unsigned blocks(int64_t n) { return (unsigned)((n + kThreads - 1) / kThreads); }
 
+// Launches of the per-step point kernels.  In 2-D programmatic ones (201^2 off-grid forward call
+// 3.57 ms against 4.40 plain, gradient 7.40 against 8.60).  In 3-D plain ones: the step's CTAs
+// fill most SMs for the whole launch, so the early CTAs of a programmatic point kernel would
+// crowd on the few SMs that hold fewer of them and, when the step ends, run there one after
+// another (90 x 75 x 110 gradient with two shots 12.1 ms plain against 14.5, 96^3 at 16th order
+// 35.7 against 40.7, 256^3 205 against 219).
+template <class... P, class... A>
+cudaError_t launch_pts(const Geom &g, void (*fn)(P...), int64_t threads, cudaStream_t s, const A &...a)
+{
+    if (g.ndim == 2) return launch_pdl(fn, dim3(blocks(threads)), dim3(kThreads), 0, s, a...);
+    fn<<<blocks(threads), kThreads, 0, s>>>(a...);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_sample_pts(const Geom &g, const float *f, const PointTaps *pts, int nshots,
@@ -188,10 +227,8 @@ cudaError_t launch_sample_pts(const Geom &g, const float *f, const PointTaps *pt
 {
     const int64_t npts = (int64_t)nshots * nrec;
     if (g.ndim == 3)
-        return launch_pdl(k_sample_pts<32, 2>, dim3(blocks(npts * 32)), dim3(kThreads), 0, s, g, f, pts, nshots,
-                          nrec, nt, n, traces, n_dev);
-    return launch_pdl(k_sample_pts<8, 1>, dim3(blocks(npts * 8)), dim3(kThreads), 0, s, g, f, pts, nshots, nrec,
-                      nt, n, traces, n_dev);
+        return launch_pts(g, k_sample_pts<32, 2>, npts * 32, s, g, f, pts, nshots, nrec, nt, n, traces, n_dev);
+    return launch_pts(g, k_sample_pts<8, 1>, npts * 8, s, g, f, pts, nshots, nrec, nt, n, traces, n_dev);
 }
 
 cudaError_t launch_inject_pts(const Geom &g, float *f, const PointTaps *pts, int npts,
@@ -201,15 +238,15 @@ cudaError_t launch_inject_pts(const Geom &g, float *f, const PointTaps *pts, int
                               const int *n_dev)
 {
     const int64_t rows = (int64_t)npts * kTaps * (g.ndim == 3 ? kTaps : 1);
-    return launch_pdl(k_inject_pts, dim3(blocks(rows)), dim3(kThreads), 0, s, g, f, pts, npts, per_shot, W,
-                      sig_z, sig_y, sig_x, q, nt, n, dt2, factor, kind, n_dev);
+    return launch_pts(g, k_inject_pts, rows, s, g, f, pts, npts, per_shot, W, sig_z, sig_y, sig_x, q, nt, n, dt2,
+                      factor, kind, n_dev);
 }
 
 cudaError_t launch_adjoint_pts(const Geom &g, const AdjointPts &a, cudaStream_t s)
 {
     const int64_t rows = (int64_t)(a.npts + a.nsrc) * kTaps * (g.ndim == 3 ? kTaps : 1);
     if (rows == 0) return cudaSuccess;
-    return launch_pdl(k_adjoint_pts, dim3(blocks(rows)), dim3(kThreads), 0, s, g, a);
+    return launch_pts(g, k_adjoint_pts, rows, s, g, a);
 }
 
 cudaError_t launch_gather_src_pts(const Geom &g, const float *f, const PointTaps *pts,

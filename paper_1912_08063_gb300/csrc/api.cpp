@@ -208,6 +208,13 @@ struct fwi_model {
     std::vector<int32_t> cl_desc_host;
     int cl_nslots = -1, cl_nt = -1;
     int resident[3] = {0, 0, 0};   // resident CTAs of the 3-D step kernel, per mode
+    // schedules of the 3-D streaming step, keyed by tile columns and resident CTAs (comparing
+    // candidate plans takes longer than a launch on the host)
+    struct PlanEntry {
+        int columns, resident, ctas;
+        int rounds, round_ctas, rem_ctas, zparts, zfirst, rem_first, rem_ppu;
+    };
+    std::vector<PlanEntry> plans;
     int resident_query[3] = {0, 0, 0};   // what the occupancy query returned (-e: error e)
     int64_t t_fwd_n = 0, t_adj_n = 0, t_st_n = 0;
     double t_fwd_ms = 0.0, t_adj_ms = 0.0, t_st_ms = 0.0;
@@ -594,6 +601,18 @@ void ensure_resident(fwi_model *m)
         }
 }
 
+// The schedule of a streaming launch over `columns` tile columns of the model's planes.
+const fwi_model::PlanEntry &plan_of(fwi_model *m, const Step3dParams &p, int columns, int resident)
+{
+    for (const auto &e : m->plans)
+        if (e.columns == columns && e.resident == resident) return e;
+    Step3dParams q = p;
+    const int ctas = plan_persistent(q, columns, resident, true);
+    m->plans.push_back({columns, resident, ctas, q.rounds, q.round_ctas, q.rem_ctas, q.zparts, q.zfirst,
+                        q.rem_first, q.rem_ppu});
+    return m->plans.back();
+}
+
 // One launch of the TMA-staged 3-D kernel (k_step3d.cu) in `mode`.
 int step3d_launch(fwi_model *m, const StepParams &p, int ns, int mode, cudaStream_t s)
 {
@@ -682,8 +701,15 @@ int step3d_launch(fwi_model *m, const StepParams &p, int ns, int mode, cudaStrea
         FWI_TRY(field_map(m, p.gacc, ns, 64, TY, &me));
     }
     const int tiles = ((g.nx + 63) / 64) * ((g.ny + TY - 1) / TY);
-    const int ctas = plan_persistent(q, tiles * ns, m->resident[mode], true);
-    FWI_CU(launch_step3d_tma(q, mode, ctas, mc, ma, mb, md, me, s));
+    const fwi_model::PlanEntry &e = plan_of(m, q, tiles * ns, m->resident[mode]);
+    q.rounds = e.rounds;
+    q.round_ctas = e.round_ctas;
+    q.rem_ctas = e.rem_ctas;
+    q.zparts = e.zparts;
+    q.zfirst = e.zfirst;
+    q.rem_first = e.rem_first;
+    q.rem_ppu = e.rem_ppu;
+    FWI_CU(launch_step3d_tma(q, mode, e.ctas, mc, ma, mb, md, me, s));
     return FWI_OK;
 }
 

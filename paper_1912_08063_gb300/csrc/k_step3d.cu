@@ -133,7 +133,7 @@ cudaError_t launch_step3d_tma(const Step3dParams &p, int mode, int ctas,
 {
     const int ty = step3d_variant(p.M, mode).ty;
     const int64_t columns = (int64_t)((p.nx + 63) / 64) * ((p.ny + ty - 1) / ty) * p.nshots;
-    bool tile_g = (int64_t)ctas > (int64_t)(kTileGParts - 1) * columns;   // ctas/columns >= 5
+    bool tile_g = (int64_t)ctas >= (int64_t)(kTileGParts - 1) * columns;
     if (const char *e = std::getenv("FWI_STEP3D_TILE_G")) tile_g = std::atoi(e) != 0;
     const Step3dKernelInfo k = kernel_info(p.M, mode, p.iso != 0, mode == kModeAdj && tile_g);
     if (!k.fn) return cudaErrorInvalidValue;

@@ -458,18 +458,20 @@ void brick_boxes(int M, int (&mid)[3], int (&arm)[3])
 }
 
 // Whether a launch takes bricks: up to the points of all shots below which they measured
-// faster than streaming.  Radius 4: forward 0.85x at 200^3 computed points, 1.1x at 192^3 and
-// 1.4x at 176^3, reverse 0.9x at 176^3 and 1.35x at 136^3.  Radius 8: 1.2 to 1.3x at 200^3, 1.03
-// to 1.13x at 224^3, 0.86 to 1.0x at 232^3.  FWI_STEP3D_BRICK=0/1 overrides; the switches that
-// choose among the streaming kernels turn bricks off.
+// faster than streaming (us, bricks / streaming).  Radius 4: forward 20.9 / 22.8 at 176^3
+// computed points and 24.9 / 24.9 at 184^3, store 24.4 / 25.3 at 168^3 and 26.9 / 26.1 at 176^3,
+// reverse 24.7 / 27.3 at 152^3, 26.0 / 26.3 at 160^3 and 37.7 / 30.3 at 168^3.  Radius 8: forward
+// 34.1 / 34.8 at 192^3 and 47.6 / 47.3 at 208^3, store 30.7 / 32.9 at 168^3 and 34.5 / 33.7 at
+// 176^3, reverse 27.4 / 32.3 at 160^3 and 40.2 / 36.7 at 168^3.  FWI_STEP3D_BRICK=0/1 overrides;
+// the switches that choose among the streaming kernels turn bricks off.
 bool step3d_use_brick(const Step3dParams &p, int mode)
 {
     if (const char *e = std::getenv("FWI_STEP3D_BRICK")) return std::atoi(e) != 0;
     for (const char *v : {"FWI_STEP3D_TMEM", "FWI_STEP3D_VARIANT", "FWI_STEP3D_HALF", "FWI_STEP3D_TILE_G"})
         if (std::getenv(v)) return false;
     const double points = (double)p.nx * p.ny * p.nz * p.nshots;
-    if (p.M == 4) return points <= (mode == kModeAdj ? 3.5e6 : 7.5e6);
-    return points <= 11.5e6;
+    if (p.M == 4) return points <= (mode == kModeStep ? 6.0e6 : mode == kModeStepStore ? 5.0e6 : 3.8e6);
+    return points <= (mode == kModeStep ? 8.5e6 : mode == kModeStepStore ? 5.2e6 : 4.3e6);
 }
 
 cudaError_t launch_step3d_brick(const Step3dParams &p, int mode, const CUtensorMap &mid,

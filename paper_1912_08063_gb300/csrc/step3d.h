@@ -29,7 +29,7 @@ struct Step3dParams {
                                   // units are numbered part-major
     int rem_first, rem_ppu;       // leftover units go to CTAs rem_first ..
                                   // rem_first + rem_ctas - 1: cut into rem_ppu aligned
-                                  // pieces each (rem_ppu > 0), or as one run cut into
+                                  // pieces each, piece-major (rem_ppu > 0), or as one run cut into
                                   // equal pieces that may cross units (rem_ppu = 0)
     float cx[kMaxM + 1], cy[kMaxM + 1], cz[kMaxM + 1], c0;
     float2 cy2[kMaxM + 1], cz2[kMaxM + 1], c02;   // the same weights as packed pairs
@@ -89,8 +89,8 @@ struct Step3dVariant {
     int half = 0;   // tensor-memory forward modes: 64 x 16 tiles, 4 warps, four CTAs per SM
 };
 // The tensor-memory reverse step takes g as a TMA tile when a launch has at least this
-// many CTAs per 64 x 32 tile column, so that its columns are cut along z into as many
-// short parts or pieces (23 to 72 planes on the 232^3 to 360^3 grids measured, 3-6 %
+// many CTAs per 64 x 32 tile column less one, so that its columns are cut along z into as
+// many short parts or pieces (23 to 72 planes on the 232^3 to 360^3 grids measured, 3-6 %
 // faster there), and stages g per thread otherwise (424^3 and up, 4-15 % faster).
 constexpr int kTileGParts = 5;
 Step3dVariant step3d_variant(int M, int mode);
@@ -164,9 +164,9 @@ __host__ __device__ inline bool schedule_segment(const Step3dParams &p, int colu
     if (rem <= 0 || kk < 0 || kk >= p.rem_ctas) return false;
     const int zb = (S - 1) * p.zfirst;            // the leftover units lie in the last part
     const int len_u = p.nz - zb;
-    if (p.rem_ppu > 0) {                          // aligned pieces, one per CTA
+    if (p.rem_ppu > 0) {                          // aligned pieces, one per CTA, piece-major
         if (idx > 0) return false;
-        const int u = first + kk / p.rem_ppu, piece = kk % p.rem_ppu;
+        const int u = first + kk % rem, piece = kk / rem;
         const int plen = (len_u + p.rem_ppu - 1) / p.rem_ppu;
         *col = u % columns;
         *z0 = zb + piece * plen;
@@ -200,23 +200,26 @@ cudaError_t launch_step2d_tile(const StepParams &p, int nshots, bool img, const 
                                cudaStream_t s);
 
 // Persistent schedule of one launch over `columns` tile columns of nz planes on
-// `resident` CTAs: rounds of whole units, then the leftover units cut along z into
-// pieces of at least 4M planes (each piece streams 2M warm-up planes).  A unit is a whole
-// column, or, with `in_step` and fewer columns than CTAs, one of S = ceil(resident /
-// columns) z-parts of a column that begin at the same z in every column: the CTAs of a
-// round then stream z in step part by part, so a tile's halo planes are still in L2 when
-// its neighbours read them.  Every launch of the step is planned in step; measured on GB300 at
-// radius 4 against plans that were not, whose neighbours stream unrelated z (us, forward /
-// store / reverse; the fields of the three grids fit in L2 one by one but not together): 216^3
-// 39.2 / 45.5 / 69.6 -> 38.4 / 43.5 / 59.2, 256^3 61 / 68 / 91 -> 53 / 58 / 74, 280^3 101 / 122 /
-// 165 -> 64 / 72 / 110; at radius 8 280^3 122 / 139 / 171 -> 87 / 97 / 103, 200^3 to 248^3 equal.  With at least as many
-// columns as CTAs, columns are cut into parts too where whole rounds of them leave less to
-// the last, partial round.  With fewer columns than CTAs the planner
-// compares equal parts (leftovers cut over all CTAs, as one run or in pieces aligned to
-// the leftover units) with longer first parts whose leftover last parts go, in aligned
-// pieces, to the CTAs that ran a last part, and keeps the one whose busiest CTA streams
-// the fewest planes (warm-up planes included).  Fills the schedule fields of p and
-// returns the grid size.
+// `resident` CTAs: rounds of whole units, then the leftover units cut along z into pieces
+// (each piece streams 2M warm-up planes).  A unit is a whole column, or, with `in_step`, one
+// of several z-parts of a column that begin at the same z in every column: the CTAs of a
+// round then stream z in step, so a tile's halo planes are still in L2 when its neighbours
+// read them.  Units are numbered part-major and pieces piece-major, so that tiles next to one
+// another in x run on CTAs next to one another.  With at least as many columns as CTAs,
+// columns are cut into parts where whole rounds of them leave less to the last, partial
+// round.  With fewer columns than CTAs the planner compares: the same number of parts of
+// every column, at most one to a CTA and none left over; S = ceil(resident / columns) equal
+// parts whose leftover last parts are cut over all CTAs; and S parts of which the first ones
+// are longer and the leftover last parts go to the CTAs that ran a last part.  It keeps the
+// one whose busiest CTA streams the fewest planes (warm-up planes included).
+// Every launch of the step is planned in step.  Measured on GB300, us per step forward /
+// store / reverse, against one run of the columns cut over all CTAs below 96 MB and no
+// candidate without leftovers: radius 4, 216^3 39.2 / 45.5 / 69.6 -> 36.2 / 41.1 / 60.2, 280^3
+// 101 / 122 / 165 -> 63 / 72 / 109, 296^3 75.9 / 85.3 / 122 -> 70.7 / 81.5 / 122; radius 8, 240^3
+// 70 / 77 / 105 -> 55.6 / 61 / 71, 280^3 122 / 139 / 171 -> 86 / 95 / 102, 440^3 263 / 296 / 361 ->
+// 257 / 286 / 348.  Pieces numbered column by column: radius 4 360^3 122 / 152 / 214 against
+// 119.6 / 137.8 / 212, 440^3 237 / 306 / 347 against 223 / 285 / 346.
+// Fills the schedule fields of p and returns the grid size.
 int plan_persistent(Step3dParams &p, int columns, int resident, bool in_step = false);
 
 }  // namespace fwi

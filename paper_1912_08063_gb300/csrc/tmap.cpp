@@ -2,6 +2,8 @@
 // point, so the library needs no libcuda link) and the persistent schedule.
 #include <cudaTypedefs.h>
 
+#include <algorithm>
+
 #include "step3d.h"
 
 namespace fwi {
@@ -140,71 +142,66 @@ int plan_persistent(Step3dParams &p, int columns, int resident, bool in_step)
     }
 
     const int S = (resident + columns - 1) / columns;   // (S - 1) columns < resident
-    if (p.nz / S < 4 * p.M) return grid;                 // parts too thin: whole columns
     Step3dParams best = p;
     int64_t best_cost = -1;
     int best_grid = grid;
-    // (a) equal parts; the leftover last parts cut over all CTAs
+    // (a) every column in the same number of pieces of at least M planes, one to a CTA
     {
-        Step3dParams q = p;
-        q.zparts = S;
-        q.zfirst = p.nz / S;
-        q.rounds = 1;
-        q.rem_first = 0;
-        q.rem_ppu = 0;
-        const long long rem_planes = (long long)(columns * S - resident) * (p.nz - (S - 1) * q.zfirst);
-        long long pieces = rem_planes / (4LL * p.M);
-        if (pieces < 1) pieces = 1;
-        if (pieces > resident) pieces = resident;
-        q.rem_ctas = rem_planes > 0 ? (int)pieces : 0;
-        const int64_t c = schedule_cost(q, columns, resident);
-        best = q;
-        best_cost = c;
-        best_grid = resident;
+        const int most = std::min(resident / columns, p.nz / p.M);
+        if (most > 1) {
+            best.zfirst = (p.nz + most - 1) / most;
+            best.zparts = (p.nz + best.zfirst - 1) / best.zfirst;
+            best.rounds = 1;
+            best.round_ctas = best_grid = columns * best.zparts;
+            best.rem_ctas = 0;
+            best_cost = schedule_cost(best, columns, best_grid);
+        }
     }
-    // (c) equal parts; the leftover last parts in aligned pieces over all CTAs
-    {
-        const int L = columns * S - resident;
-        const int ppu = L > 0 ? resident / L : 0;
-        if (ppu >= 1) {
-            Step3dParams q = best;
+    if (p.nz / S >= 4 * p.M) {
+        // (b) equal parts; the L leftover last parts in aligned pieces over all CTAs
+        {
+            const int L = columns * S - resident, ppu = L > 0 ? resident / L : 0;
+            Step3dParams q = p;
+            q.zparts = S;
+            q.zfirst = p.nz / S;
+            q.rounds = 1;
             q.rem_first = 0;
             q.rem_ppu = ppu;
             q.rem_ctas = L * ppu;
             const int64_t c = schedule_cost(q, columns, resident);
-            if (c < best_cost) {
+            if (best_cost < 0 || c < best_cost) {
                 best = q;
                 best_cost = c;
+                best_grid = resident;
             }
         }
-    }
-    // (b) longer first parts; the L leftover last parts go in ppu aligned pieces to the
-    // qn CTAs that ran a last part, with lengths that balance both kinds of CTA:
-    // first part + 2M = last part + 2M + last part / ppu + 2M
-    {
-        const int qn = resident - (S - 1) * columns, L = columns - qn;
-        const int ppu = L > 0 ? qn / L : 0;
-        if (L > 0 && ppu >= 1) {
-            const double ll = (double)(p.nz - 2 * p.M * (S - 1)) / ((S - 1) * (1.0 + 1.0 / ppu) + 1.0);
-            Step3dParams q = p;
-            q.zparts = S;
-            q.zfirst = (int)((p.nz - ll) / (S - 1) + 0.5);
-            const int last = p.nz - (S - 1) * q.zfirst;
-            if (last >= 2 * p.M && q.zfirst >= 4 * p.M) {
-                q.rounds = 1;
-                q.rem_first = (S - 1) * columns;
-                q.rem_ppu = ppu;
-                q.rem_ctas = L * ppu;
-                const int64_t c = schedule_cost(q, columns, resident);
-                if (c < best_cost) {
-                    best = q;
-                    best_cost = c;
+        // (c) longer first parts; the L leftover last parts go in ppu aligned pieces to the
+        // qn CTAs that ran a last part, with lengths that balance both kinds of CTA:
+        // first part + 2M = last part + 2M + last part / ppu + 2M
+        {
+            const int qn = resident - (S - 1) * columns, L = columns - qn;
+            const int ppu = L > 0 ? qn / L : 0;
+            if (L > 0 && ppu >= 1) {
+                const double ll = (double)(p.nz - 2 * p.M * (S - 1)) / ((S - 1) * (1.0 + 1.0 / ppu) + 1.0);
+                Step3dParams q = p;
+                q.zparts = S;
+                q.zfirst = (int)((p.nz - ll) / (S - 1) + 0.5);
+                const int last = p.nz - (S - 1) * q.zfirst;
+                if (last >= 2 * p.M && q.zfirst >= 4 * p.M) {
+                    q.rounds = 1;
+                    q.rem_first = (S - 1) * columns;
+                    q.rem_ppu = ppu;
+                    q.rem_ctas = L * ppu;
+                    const int64_t c = schedule_cost(q, columns, resident);
+                    if (best_cost < 0 || c < best_cost) {
+                        best = q;
+                        best_cost = c;
+                        best_grid = resident;
+                    }
                 }
             }
         }
     }
-    const Step3dParams keep = p;
-    p = keep;
     p.zparts = best.zparts;
     p.zfirst = best.zfirst;
     p.rounds = best.rounds;

@@ -336,58 +336,30 @@ int set_velocity(fwi_model *m, const float *vp, cudaStream_t s)
     return FWI_OK;
 }
 
-// Kaiser-windowed sinc weights of an off-grid point along one axis (Hicks 2002,
-// Geophysics 67(1)): the 8 nodes first .. first + 7 around the computed-grid coordinate p
-// get sinc(x - p) I0(6.31 sqrt(1 - ((x - p) / 4)^2)) / I0(6.31).  At integer p the weights
-// are the delta at p.
-void sinc_weights(double p, int32_t *first, float *w)
-{
-    auto i0 = [](double x) {   // modified Bessel function of order 0, power series
-        double term = 1.0, total = 1.0;
-        const double q = x * x / 4.0;
-        for (int k = 1; k < 400 && term > 1e-18 * total; ++k) {
-            term = term * q / ((double)k * k);
-            total += term;
-        }
-        return total;
-    };
-    const double kb = 6.31, half = kTaps / 2, pi = 3.14159265358979323846;
-    const double fl = std::floor(p);
-    *first = (int32_t)fl - (int32_t)half + 1;
-    const double norm = i0(kb);
-    for (int k = 0; k < kTaps; ++k) {
-        const double t = (double)(*first + k) - p;
-        double sinc;
-        if (t == std::floor(t)) sinc = (t == 0.0) ? 1.0 : 0.0;
-        else sinc = std::sin(pi * t) / (pi * t);
-        const double r = t / half;
-        const double win = (r >= -1.0 && r <= 1.0) ? i0(kb * std::sqrt(1.0 - r * r)) / norm : 0.0;
-        w[k] = (float)(sinc * win);
-    }
-}
-
-// Taps of the off-grid point at physical-grid position pos (z, y, x); false when a tap
-// would fall outside the computed grid.
-bool point_taps(const fwi_model *m, const double *pos, PointTaps *out)
+// Whether the taps of an off-grid point at physical-grid position pos (z, y, x) lie in the
+// computed grid (k_points.cu computes them).
+bool taps_inside(const fwi_model *m, const double *pos)
 {
     const int nby = m->ndim == 3 ? m->nb : 0;
     const double c[3] = {pos[0] + m->nb, pos[1] + nby, pos[2] + m->nb};
     const int64_t n[3] = {m->g.nz, m->g.ny, m->g.nx};
-    int32_t first[3] = {0, 0, 0};
     for (int a = 0; a < 3; ++a) {
-        if (a == 1 && m->ndim == 2) {
-            out->w[kTaps] = 1.0f;
-            for (int k = 1; k < kTaps; ++k) out->w[kTaps + k] = 0.0f;
-            continue;
-        }
-        sinc_weights(c[a], &first[a], out->w + a * kTaps);
-        if (first[a] < 0 || first[a] + kTaps > n[a]) return false;
+        if (a == 1 && m->ndim == 2) continue;
+        const int64_t first = (int64_t)std::floor(c[a]) - kTaps / 2 + 1;
+        if (first < 0 || first + kTaps > n[a]) return false;
     }
-    out->z0 = first[0];
-    out->y0 = first[1];
-    out->x0 = first[2];
-    out->pad = 0;
     return true;
+}
+
+// The taps of `n` off-grid points, in dst; the positions lie behind them meanwhile.
+int upload_points(fwi_model *m, DevBuf &dst, const double *pos, size_t n, cudaStream_t s)
+{
+    static_assert(sizeof(PointTaps) % sizeof(double) == 0, "positions lie behind the taps");
+    FWI_TRY(dst.ensure(n * (sizeof(PointTaps) + 3 * sizeof(double))));
+    double *at = (double *)(dst.as<PointTaps>() + n);
+    FWI_CU(cudaMemcpyAsync(at, pos, n * 3 * sizeof(double), cudaMemcpyHostToDevice, s));
+    FWI_LAUNCH(m, launch_point_taps(m->g, at, (int64_t)n, m->nb, dst.as<PointTaps>(), s));
+    return FWI_OK;
 }
 
 int validate_acq(const fwi_model *m, const fwi_acq *a)
@@ -407,16 +379,15 @@ int validate_acq(const fwi_model *m, const fwi_acq *a)
         if (m->ndim == 3) return p[1] >= 0.0 && p[1] <= (double)(m->np[1] - 1);
         return p[1] == 0.0;
     };
-    PointTaps t;
     if (a->src_pos)
         for (int s = 0; s < a->nshots; ++s)
-            if (!inside_pos(a->src_pos + 3 * s) || !point_taps(m, a->src_pos + 3 * s, &t))
+            if (!inside_pos(a->src_pos + 3 * s) || !taps_inside(m, a->src_pos + 3 * s))
                 return fail(FWI_ERR_ARG, "source position " + std::to_string(s) +
                                              " outside the grid or its taps outside the "
                                              "sponge (nb >= 4 needed near the edges)");
     if (a->rec_pos)
         for (int64_t i = 0; i < (int64_t)a->nshots * a->nrec; ++i)
-            if (!inside_pos(a->rec_pos + 3 * i) || !point_taps(m, a->rec_pos + 3 * i, &t))
+            if (!inside_pos(a->rec_pos + 3 * i) || !taps_inside(m, a->rec_pos + 3 * i))
                 return fail(FWI_ERR_ARG, "receiver position " + std::to_string(i) +
                                              " outside the grid or its taps outside the "
                                              "sponge (nb >= 4 needed near the edges)");
@@ -482,18 +453,13 @@ int ensure_workspace(fwi_model *m, const fwi_acq *a, bool grad, cudaStream_t s)
                 m->og_src == og_s && m->og_rec == og_r;
     if (!same) {
         std::vector<int64_t> so(ns, 0), ro((size_t)ns * nr, 0);
-        std::vector<PointTaps> sp, rp;
         if (og_s) {
-            sp.resize(ns);
-            for (int i = 0; i < ns; ++i) point_taps(m, a->src_pos + 3 * i, &sp[i]);
-            FWI_TRY(m->src_pts.ensure(sp.size() * sizeof(PointTaps)));
+            FWI_TRY(upload_points(m, m->src_pts, a->src_pos, (size_t)ns, s));
         } else {
             for (int i = 0; i < ns; ++i) so[i] = node_offset(m, a->src + 3 * i);
         }
         if (og_r) {
-            rp.resize((size_t)ns * nr);
-            for (size_t i = 0; i < rp.size(); ++i) point_taps(m, a->rec_pos + 3 * i, &rp[i]);
-            FWI_TRY(m->rec_pts.ensure(rp.size() * sizeof(PointTaps)));
+            FWI_TRY(upload_points(m, m->rec_pts, a->rec_pos, (size_t)ns * nr, s));
         } else {
             for (size_t i = 0; i < (size_t)ns * nr; ++i) ro[i] = node_offset(m, a->rec + 3 * i);
         }
@@ -501,12 +467,6 @@ int ensure_workspace(fwi_model *m, const fwi_acq *a, bool grad, cudaStream_t s)
                                cudaMemcpyHostToDevice, s));
         FWI_CU(cudaMemcpyAsync(m->rec_off.p, ro.data(), ro.size() * sizeof(int64_t),
                                cudaMemcpyHostToDevice, s));
-        if (og_s)
-            FWI_CU(cudaMemcpyAsync(m->src_pts.p, sp.data(), sp.size() * sizeof(PointTaps),
-                                   cudaMemcpyHostToDevice, s));
-        if (og_r)
-            FWI_CU(cudaMemcpyAsync(m->rec_pts.p, rp.data(), rp.size() * sizeof(PointTaps),
-                                   cudaMemcpyHostToDevice, s));
         // receivers on one plane at distinct nodes: map them for the step kernels
         m->rec_fuse_z = -1;
         std::vector<int32_t> rmap;

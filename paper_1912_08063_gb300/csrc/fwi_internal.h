@@ -99,6 +99,10 @@ struct PointTaps {
 };
 
 // ---- off-grid points (k_points.cu) ----
+// The taps of npts points at physical-grid positions pos[i] = (z, y, x), on a grid with a
+// sponge of nb nodes.
+cudaError_t launch_point_taps(const Geom &g, const double *pos, int64_t npts, int nb, PointTaps *out,
+                              cudaStream_t s);
 cudaError_t launch_sample_pts(const Geom &g, const float *f, const PointTaps *pts, int nshots,
                               int nrec, int nt, int n, float *traces, cudaStream_t s,
                               const int *n_dev = nullptr);

@@ -58,3 +58,34 @@ def test_receiver_samples_at_integer_positions(shape):
     pos = m.forward(fwi.Acquisition(src, rec_pos=rec.astype(np.float64)), wav)
     assert torch.equal(node, pos) and node.abs().max() > 0
     m.close()
+
+
+@pytest.mark.parametrize("shape", [(40, 150), (18, 25, 40)])
+def test_tap_weights_match_the_oracle(shape):
+    """Samples of the last state at the corners, edges and random positions of the grid, against
+    the oracle's taps applied to that state."""
+    import oracle
+    from paper_1912_08063_gb300 import fwi
+    rng = np.random.default_rng(4)
+    v = rng.uniform(1600.0, 4400.0, shape).astype(np.float32)
+    h, nt, nb = 10.0, 60, 5
+    dt = 0.35 * h / 4600.0
+    hi = np.array(shape if len(shape) == 3 else (shape[0], 1, shape[1]))
+    src = (hi // 2)[None].astype(np.int32)
+    frac = np.array([[0, 0, 0], [1, 1, 1], [0, 1, 0.5], [1, 0, 0.25]] + rng.random((40, 3)).tolist())
+    pos = frac * (hi - 1)
+    pos[10:20] = np.floor(pos[10:20]) + [0.5, 0.0 if hi[1] == 1 else 0.5, 1e-9]
+    pos = np.minimum(pos, hi - 1)
+    wav = torch.from_numpy(synth.ricker(50.0, dt, nt)[None].astype(np.float32)).cuda()
+    m = fwi.FwiModel(torch.from_numpy(v).cuda(), h, dt, nt, nb=nb, sponge_vref=4600.0)
+    tr, fin = m.forward(fwi.Acquisition(src, rec_pos=pos), wav, final_state=True)
+    u = fin.cpu().numpy()[0, 0].astype(np.float64).ravel()   # u^nt, the last trace row's state
+    got = tr.cpu().numpy()[0, -1]
+    for p, g in zip(pos, got):
+        idx, w = oracle.point_taps(shape, p if len(shape) == 3 else p[[0, 2]], nb=nb)
+        ref, mag = np.sum(w * u[idx]), np.sum(np.abs(w * u[idx]))
+        # each weight is a product of FP32-rounded factors, the sum is in FP32: 64 or 512 terms
+        # in chains of at most 8 and a tree of at most 6, and three roundings a weight
+        assert abs(g - ref) <= (8 + 6 + 3) * 2.0 ** -24 * mag * 2 + 1e-30
+    assert np.abs(got).max() > 0
+    m.close()

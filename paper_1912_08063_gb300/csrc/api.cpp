@@ -208,10 +208,10 @@ struct fwi_model {
     std::vector<int32_t> cl_desc_host;
     int cl_nslots = -1, cl_nt = -1;
     int resident[3] = {0, 0, 0};   // resident CTAs of the 3-D step kernel, per mode
-    // schedules of the 3-D streaming step, keyed by tile columns, CTAs and `share` (comparing
+    // schedules of the 3-D streaming step, keyed by tile columns and resident CTAs (comparing
     // candidate plans takes longer than a launch on the host)
     struct PlanEntry {
-        int columns, resident, share, ctas;
+        int columns, resident, ctas;
         int rounds, round_ctas, rem_ctas, zparts, zfirst, rem_first, rem_ppu;
     };
     std::vector<PlanEntry> plans;
@@ -562,13 +562,13 @@ void ensure_resident(fwi_model *m)
 }
 
 // The schedule of a streaming launch over `columns` tile columns of the model's planes.
-const fwi_model::PlanEntry &plan_of(fwi_model *m, const Step3dParams &p, int columns, int resident, bool share)
+const fwi_model::PlanEntry &plan_of(fwi_model *m, const Step3dParams &p, int columns, int resident)
 {
     for (const auto &e : m->plans)
-        if (e.columns == columns && e.resident == resident && e.share == share) return e;
+        if (e.columns == columns && e.resident == resident) return e;
     Step3dParams q = p;
-    const int ctas = plan_persistent(q, columns, resident, true, share);
-    m->plans.push_back({columns, resident, share, ctas, q.rounds, q.round_ctas, q.rem_ctas, q.zparts, q.zfirst,
+    const int ctas = plan_persistent(q, columns, resident, true);
+    m->plans.push_back({columns, resident, ctas, q.rounds, q.round_ctas, q.rem_ctas, q.zparts, q.zfirst,
                         q.rem_first, q.rem_ppu});
     return m->plans.back();
 }
@@ -650,8 +650,7 @@ int step3d_launch(fwi_model *m, const StepParams &p, int ns, int mode, cudaStrea
         FWI_CU(launch_step3d_brick(q, mode, mid, arm, s));
         return FWI_OK;
     }
-    const Step3dVariant v = step3d_variant(g.M, mode);
-    const int TY = v.ty;
+    const int TY = step3d_variant(g.M, mode).ty;
     CUtensorMap mc, ma, mb, md, me;
     FWI_TRY(field_map(m, p.cur, ns, 64 + 2 * g.M, TY + 2 * g.M, &mc));
     FWI_TRY(field_map(m, p.prev, ns, 64, TY, &ma));
@@ -662,7 +661,7 @@ int step3d_launch(fwi_model *m, const StepParams &p, int ns, int mode, cudaStrea
         FWI_TRY(field_map(m, p.gacc, ns, 64, TY, &me));
     }
     const int tiles = ((g.nx + 63) / 64) * ((g.ny + TY - 1) / TY);
-    const fwi_model::PlanEntry &e = plan_of(m, q, tiles * ns, m->resident[mode], g.M == 4 && mode == kModeAdj && !v.tm);
+    const fwi_model::PlanEntry &e = plan_of(m, q, tiles * ns, m->resident[mode]);
     q.rounds = e.rounds;
     q.round_ctas = e.round_ctas;
     q.rem_ctas = e.rem_ctas;

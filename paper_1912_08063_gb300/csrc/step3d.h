@@ -219,11 +219,7 @@ cudaError_t launch_step2d_tile(const StepParams &p, int nshots, bool img, const 
 // 70 / 77 / 105 -> 55.6 / 61 / 71, 280^3 122 / 139 / 171 -> 86 / 95 / 102, 440^3 263 / 296 / 361 ->
 // 257 / 286 / 348.  Pieces numbered column by column: radius 4 360^3 122 / 152 / 214 against
 // 119.6 / 137.8 / 212, 440^3 237 / 306 / 347 against 223 / 285 / 346.
-// share: also consider the first candidate with shorter parts, whose last planes the CTAs left
-// over take, several columns each.  For the register-queue reverse step at radius 4, whose CTAs
-// are bound by their arithmetic: 296^3 121 -> 117 us, 360^3 212 -> 198, 280^3 109.5 -> 106.6; the
-// other steps are bound by memory and lose by it (radius 4 store at 360^3 142 -> 150 us).
 // Fills the schedule fields of p and returns the grid size.
-int plan_persistent(Step3dParams &p, int columns, int resident, bool in_step = false, bool share = false);
+int plan_persistent(Step3dParams &p, int columns, int resident, bool in_step = false);
 
 }  // namespace fwi

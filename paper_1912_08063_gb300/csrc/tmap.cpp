@@ -83,7 +83,7 @@ static int64_t schedule_cost(const Step3dParams &p, int columns, int grid)
     return worst;
 }
 
-int plan_persistent(Step3dParams &p, int columns, int resident, bool in_step, bool share)
+int plan_persistent(Step3dParams &p, int columns, int resident, bool in_step)
 {
     if (resident < 1) resident = 1;
     if (columns < 1) columns = 1;
@@ -155,34 +155,6 @@ int plan_persistent(Step3dParams &p, int columns, int resident, bool in_step, bo
             best.round_ctas = best_grid = columns * best.zparts;
             best.rem_ctas = 0;
             best_cost = schedule_cost(best, columns, best_grid);
-        }
-    }
-    // (share) the parts of (a) made shorter, and the last planes of every column shared by the
-    // CTAs that (a) leaves over, whole columns at a time
-    const int q = resident / columns, left = resident - q * columns;
-    if (share && q > 1 && left > 0) {
-        const int each = (columns + left - 1) / left;
-        int len = 0;
-        for (int last = 1; last < p.nz / 2; ++last) {   // as many planes as those CTAs have time for
-            const int n = (p.nz - last + q - 1) / q;
-            if (each * (p.nz - q * n + 2 * p.M) > n + 2 * p.M) break;
-            len = n;
-        }
-        if (len >= p.M && p.nz > q * len) {
-            Step3dParams b = p;
-            b.zfirst = len;
-            b.zparts = q + 1;
-            b.rounds = 1;
-            b.round_ctas = b.rem_first = q * columns;
-            b.rem_ppu = 0;
-            b.rem_ctas = (columns + each - 1) / each;
-            const int grid_b = b.round_ctas + b.rem_ctas;
-            const int64_t c = schedule_cost(b, columns, grid_b);
-            if (best_cost < 0 || c < best_cost) {
-                best = b;
-                best_cost = c;
-                best_grid = grid_b;
-            }
         }
     }
     if (p.nz / S >= 4 * p.M) {

@@ -21,7 +21,12 @@
 //   one shot of 241 x 241, radius 4:   12.7 /  14.9 /  20.6  ->   6.2 /  6.3 /   8.0
 // (5.4 / 5.3 / 6.1 TB/s on the first line; the last two hold a few us of event overhead).
 // What bounds it: the latency of a CTA's loads.  Its load phase and its arithmetic do not
-// overlap, what hides one is the SM's other CTAs, and registers cap those.
+// overlap, what hides one is the SM's other CTAs, and registers cap those: 14.4 warps an SM,
+// issue slots 48 % and the L1 data pipe 49 % busy.  It is not DRAM: 16 shots, whose fields stay
+// in L2, take the same time per point (18.5 us).  A persistent pipeline of 128 x 32 tiles, all
+// operands by TMA in a ring of two stages, two CTAs of 8 warps an SM, gave the forward step 70.3
+// -> 66.4 us but the storing one 84.2 -> 84.4, radius 8 76.0 -> 87.6 and 16 shots 18.5 -> 21.1;
+// rows of a later tile prefetched into L2 gave 2 % forward and took 2 % in reverse.
 //
 // Tile: two warps of 4 rows, eight CTAs per SM (forward modes), or of 3 rows (reverse, which
 // holds twice the operands).  Measured at radius 4, forward / store / reverse: 2 warps x 2

@@ -20,13 +20,21 @@ namespace fwi {
 // per tile column, kTileGParts).  By default, as measured on GB300: the
 // tensor-memory kernel in every mode at radius 8, and at radius 4 in the forward modes
 // (forward 0.090 -> 0.087 ms, forward + store 0.108 -> 0.085 ms at 296^3) but not in the
-// reverse mode (0.1165 against 0.1194 ms).  The register-queue kernel at radius 8 shifts
+// reverse mode.  That runs the register queue with one row per thread: its CTAs' shared memory
+// admits two of them per SM, and with two rows per thread those held 8 warps, issuing 39 % of
+// the time; one row makes them 16 (same sums in the same order).  us, two rows / one row: 184^3
+// 38.1 / 33.9, 216^3 60.2 / 53.6, 256^3 74.2 / 71.2, 296^3 121 / 109, 360^3 212 / 188, 440^3 345 /
+// 331; a queue shifted every 1, 3 or 4 planes instead of 2 gains nothing (296^3 110.1, 107.4,
+// 108.3 against 107.2).  The register-queue kernel at radius 8 shifts
 // its queue every 2 planes and takes the packed x-sums in all modes (measured fastest
 // against U = 3 and scalar x-sums).
 Step3dVariant step3d_variant(int M, int mode)
 {
     Step3dVariant v = M == 8 ? Step3dVariant{32, 2, 2, 2, 1, 1, 1} : Step3dVariant{16, 2, 3, 2, 0, 0, 0};
-    if (M == 4) v.tm = mode != kModeAdj;
+    if (M == 4) {
+        v.tm = mode != kModeAdj;
+        if (mode == kModeAdj) v.ry = 1;
+    }
     if (const char *e = std::getenv("FWI_STEP3D_TMEM")) v.tm = std::atoi(e) != 0;
     if (const char *e = std::getenv("FWI_STEP3D_VARIANT")) {
         int ty, ry, pf, un, opt, optr;

@@ -719,25 +719,31 @@ constexpr int adj_prefetch()
     return P;
 }
 
-// Kernel, block size and dynamic shared memory of one configuration in `mode`.
+// Kernel, block size and dynamic shared memory of one configuration's reverse mode.
+template <int M, int TY, int RY, int P, int U, int F>
+Step3dKernelInfo adj_info()
+{
+    constexpr int PA = adj_prefetch<M, TY, RY, P, U, F>();
+    using C = Cfg<M, TY, RY, PA, U, F, 4>;
+    static_assert(C::SMEM <= 232448, "shared memory of the reverse-step kernel");
+    Step3dKernelInfo k;
+    k.fn = (Step3dKernel)k_step3d_tma<M, TY, RY, PA, U, F, kModeAdj>;
+    k.threads = C::NT;
+    k.smem = C::SMEM;
+    return k;
+}
+
+// The same in `mode`.
 template <int M, int TY, int RY, int P, int U, int F>
 Step3dKernelInfo kernel_info(int mode)
 {
+    if (mode == kModeAdj) return adj_info<M, TY, RY, P, U, F>();
     Step3dKernelInfo k;
-    if (mode == kModeStep || mode == kModeStepStore) {
-        using C = Cfg<M, TY, RY, P, U, F, 2>;
-        k.fn = mode == kModeStep ? (Step3dKernel)k_step3d_tma<M, TY, RY, P, U, F, kModeStep>
-                                 : (Step3dKernel)k_step3d_tma<M, TY, RY, P, U, F, kModeStepStore>;
-        k.threads = C::NT;
-        k.smem = C::SMEM;
-    } else {
-        constexpr int PA = adj_prefetch<M, TY, RY, P, U, F>();
-        using C = Cfg<M, TY, RY, PA, U, F, 4>;
-        static_assert(C::SMEM <= 232448, "shared memory of the reverse-step kernel");
-        k.fn = (Step3dKernel)k_step3d_tma<M, TY, RY, PA, U, F, kModeAdj>;
-        k.threads = C::NT;
-        k.smem = C::SMEM;
-    }
+    using C = Cfg<M, TY, RY, P, U, F, 2>;
+    k.fn = mode == kModeStep ? (Step3dKernel)k_step3d_tma<M, TY, RY, P, U, F, kModeStep>
+                             : (Step3dKernel)k_step3d_tma<M, TY, RY, P, U, F, kModeStepStore>;
+    k.threads = C::NT;
+    k.smem = C::SMEM;
     return k;
 }
 

@@ -16,10 +16,13 @@
 //
 // Measured on GB300 against the streaming kernels, us per launch with about 4 us of event
 // overhead, forward / forward + store / reverse (computed cubes, 40 cells wider than named):
-//   radius 4:   56^3  22.7 / 25.6 / 26.3 ->  8.9 /  9.2 / 10.4   96^3  23.7 / 26.8 / 28.4 -> 14.4 / 15.6 / 21.0
-//              128^3  31.6 / 35.0 / 34.6 -> 19.1 / 22.9 / 38.9  160^3  36.7 / 41.1 / 55.3 -> 37.6 / 43.7 / 64.6
-//   radius 8:   56^3  38.8 / 43.4 / 56.3 -> 10.6 / 10.7 / 11.4   96^3  45.5 / 49.2 / 63.0 -> 18.1 / 20.1 / 24.4
-//              160^3  60.1 / 65.1 / 84.4 -> 46.4 / 54.4 / 68.7  224^3  86.0 /101.3 /145.5 -> 91.8 /109.2 /140.4
+//   radius 4:   56^3  14.0 / 14.6 / 13.3 ->  8.9 /  9.6 / 10.2   96^3  18.6 / 20.6 / 22.4 -> 14.5 / 16.8 / 20.2
+//              120^3  20.0 / 21.6 / 24.5 -> 16.5 / 19.1 / 26.1  160^3  32.9 / 38.7 / 49.8 -> 38.1 / 45.4 / 61.7
+//   radius 8:   56^3  18.7 / 20.7 / 24.2 -> 10.5 / 10.8 / 10.6   96^3  27.0 / 29.0 / 31.3 -> 17.1 / 20.4 / 23.1
+//              120^3  28.5 / 30.7 / 32.3 -> 21.3 / 24.9 / 27.4  160^3  46.0 / 51.0 / 55.6 -> 45.9 / 57.8 / 66.5
+// (before the streaming plans of step3d.h cut columns into equal parts the radius-8 streaming
+// steps took 45.5 / 49.2 / 63.0 at 96^3).  What bounds it at 96^3 is latency: issue slots 35 %
+// busy with 11 warps an SM, the warps waiting on global loads and shared memory.
 // Brick: 32 x 8 x 8 by four warps (96^3 radius 8 18.8 / 20.4 / 25.5, 160^3 46.5 / 52.0 / 74.4),
 // 32 x 16 x 8 (19.6 / 21.0 / 28.4, 52.0 / 56.4 / 91.9), 32 x 8 x 16 (19.7 / 21.1 / 28.4, 50.7 /
 // 55.5 / 93.6) read fewer halo floats but leave fewer, larger CTAs and were no faster; one
@@ -460,7 +463,7 @@ void brick_boxes(int M, int (&mid)[3], int (&arm)[3])
 // Whether a launch takes bricks: up to the points of all shots below which they measured
 // faster than streaming (us, bricks / streaming).  Radius 4: forward 20.9 / 22.8 at 176^3
 // computed points and 24.9 / 24.9 at 184^3, store 24.4 / 25.3 at 168^3 and 26.9 / 26.1 at 176^3,
-// reverse 24.7 / 27.3 at 152^3, 26.0 / 26.3 at 160^3 and 37.7 / 30.3 at 168^3.  Radius 8: forward
+// reverse 20.2 / 22.4 at 136^3, 22.2 / 22.3 at 144^3 and 24.9 / 24.5 at 152^3.  Radius 8: forward
 // 34.1 / 34.8 at 192^3 and 47.6 / 47.3 at 208^3, store 30.7 / 32.9 at 168^3 and 34.5 / 33.7 at
 // 176^3, reverse 27.4 / 32.3 at 160^3 and 40.2 / 36.7 at 168^3.  FWI_STEP3D_BRICK=0/1 overrides;
 // the switches that choose among the streaming kernels turn bricks off.
@@ -470,7 +473,7 @@ bool step3d_use_brick(const Step3dParams &p, int mode)
     for (const char *v : {"FWI_STEP3D_TMEM", "FWI_STEP3D_VARIANT", "FWI_STEP3D_HALF", "FWI_STEP3D_TILE_G"})
         if (std::getenv(v)) return false;
     const double points = (double)p.nx * p.ny * p.nz * p.nshots;
-    if (p.M == 4) return points <= (mode == kModeStep ? 6.0e6 : mode == kModeStepStore ? 5.0e6 : 3.8e6);
+    if (p.M == 4) return points <= (mode == kModeStep ? 6.0e6 : mode == kModeStepStore ? 5.0e6 : 3.0e6);
     return points <= (mode == kModeStep ? 8.5e6 : mode == kModeStepStore ? 5.2e6 : 4.3e6);
 }
 

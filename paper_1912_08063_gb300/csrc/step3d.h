@@ -212,7 +212,8 @@ cudaError_t launch_step2d_tile(const StepParams &p, int nshots, bool img, const 
 // parts whose leftover last parts are cut over all CTAs; and S parts of which the first ones
 // are longer and the leftover last parts go to the CTAs that ran a last part.  It keeps the
 // one whose busiest CTA streams the fewest planes (warm-up planes included).
-// Every launch of the step is planned in step.  Measured on GB300, us per step forward /
+// Every launch of the step is planned in step.  Measured on GB300 (the radius-4 reverse step
+// still with two rows per thread), us per step forward /
 // store / reverse, against one run of the columns cut over all CTAs below 96 MB and no
 // candidate without leftovers: radius 4, 216^3 39.2 / 45.5 / 69.6 -> 36.2 / 41.1 / 60.2, 280^3
 // 101 / 122 / 165 -> 63 / 72 / 109, 296^3 75.9 / 85.3 / 122 -> 70.7 / 81.5 / 122; radius 8, 240^3

@@ -1768,7 +1768,7 @@ bool job_batchable(const Job *j)
 // Whether the job's turns are runs of steps on chip.
 bool job_onchip(const Job *j) { return j->kind == 0 ? j->f.onchip > 0 : j->gj.on_fwd > 0; }
 
-int job_batch_entry(Job *j, Batch2dEntry *e, int zchunk)
+int job_batch_entry(Job *j, Batch2dEntry *e)
 {
     if (!job_batchable(j)) return fail(FWI_ERR_ARG, "job not eligible for the shared launch");
     const FwdJob &f = j->f;
@@ -1789,8 +1789,6 @@ int job_batch_entry(Job *j, Batch2dEntry *e, int zchunk)
         }
     }
     e->p = f.p;
-    e->p.zchunk = zchunk;
-    e->p.nzchunks = (m->g.nz + zchunk - 1) / zchunk;
     e->p.n_dev = nullptr;
     e->p.err = f.m->d_flag;
     e->p.rec_tr = f.tr;
@@ -1800,7 +1798,8 @@ int job_batch_entry(Job *j, Batch2dEntry *e, int zchunk)
     e->u0 = f.uc;
     e->u1 = f.up;
     e->n0 = f.n;
-    e->xtiles = (m->g.nx + 255) / 256;
+    e->xtiles = (m->g.nx + kMultiCols - 1) / kMultiCols;
+    e->ztiles = (m->g.nz + kMultiRows - 1) / kMultiRows;
     e->rec_off = m->rec_off.as<int64_t>();
     e->traces = f.tr;
     e->nrec = f.nr;

@@ -62,8 +62,6 @@ struct StepParams {
     int64_t aux_stride;       // elements per shot
     const float *aux_scale;   // per shot at [2 s], or nullptr (scale 1)
     float *gacc;              // imaging only: gradient accumulator
-    int zchunk;               // shared 2-D launch: rows per work item along z
-    int nzchunks;
     // nullable, forward step only: a checkpoint store of this step's input pair
     // (cur = u^n, prev = u^{n-1}) written from the epilogue before prev is overwritten, in
     // the encode kernel's format (component a = u^n, d = u^n - u^{n-1}, or the FP32 pair)
@@ -137,10 +135,10 @@ cudaError_t launch_gather_src_pts(const Geom &g, const float *f, const PointTaps
 // k launches of each kernel (step t = 0 .. k - 1).
 struct Batch2dEntry {
     StepParams p;             // the request's step parameters (g, c, W, sig, src_off,
-                              // wavelet, nt, dt2, zchunk, nzchunks; cur/prev/n unused)
+                              // wavelet, nt, dt2; cur/prev/n unused)
     float *u0, *u1;           // u^{n0} and u^{n0 - 1} at the tick's start
     int n0;                   // step index at the tick's start
-    int xtiles;               // work items: xtiles x p.nzchunks
+    int xtiles, ztiles;       // work items: tiles of kMultiCols x kMultiRows
     int work0, rec0;          // first work item and first receiver of the entry
     const int64_t *rec_off;   // [nrec] receiver offsets in the field
     float *traces;            // [nt][nrec]
@@ -149,9 +147,10 @@ struct Batch2dEntry {
                               // step samples them (rec_z >= 0)
     int rec_z, rec_x0;        // receivers on row rec_z, columns rec_x0 .. rec_x0 + nrec - 1
                               // (rec_z = -1: any other layout)
-    int pad[2];
+    int pad;
 };
 constexpr int kBatch2dMax = 64;
+constexpr int kMultiCols = 128, kMultiRows = 8;   // tile of a work item
 struct Batch2d {
     int count, total_work, total_rec, pad;   // total_rec: receivers of the sampling kernel
     Batch2dEntry e[kBatch2dMax];

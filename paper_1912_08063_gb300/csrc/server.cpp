@@ -41,7 +41,7 @@ namespace fwi {
 struct Job;
 bool job_batchable(const Job *j);
 bool job_onchip(const Job *j);
-int job_batch_entry(Job *j, Batch2dEntry *e, int zchunk);
+int job_batch_entry(Job *j, Batch2dEntry *e);
 int job_batch_moved(Job *j, int steps, bool *done);
 Job *job_forward(fwi_model *m, const fwi_acq *acq, const float *wavelets, cudaStream_t s, int *rc);
 Job *job_gradient(fwi_model *m, const fwi_acq *acq, const float *wavelets, const float *d_obs,
@@ -99,7 +99,6 @@ struct Pool {
     bool failed = false;               // set-up failed: requests run on their own streams
 };
 
-constexpr int kPoolZChunk = 128;   // most rows per work item of the multi-request step
 constexpr int kPools = 4;          // shared-launch pools per stencil radius
 // Cluster pools take the grids that fit on chip and advance them by at least kClusterTick
 // steps per tick (the states stay on chip for the whole launch).
@@ -335,7 +334,7 @@ extern "C" int fwi_serve(const fwi_request *reqs, int32_t n, const fwi_serve_opt
                 fwi::Batch2dEntry probe;
                 int kind = 0;
                 const int C = cl_size[ri];
-                if (C > 0 && fwi::job_batch_entry(free_slot->job, &probe, 64) == FWI_OK &&
+                if (C > 0 && fwi::job_batch_entry(free_slot->job, &probe) == FWI_OK &&
                     probe.p.rec_map && fwi::onchip2d_fits(probe.p.g, C, 0))
                     kind = 1;
                 const int pi = (kind * 2 + ri) * kPools + (rr++ % kPools);
@@ -428,25 +427,15 @@ extern "C" int fwi_serve(const fwi_request *reqs, int32_t n, const fwi_serve_opt
             }
             fwi::Batch2d *h = pl.host[pl.buf];
             int work = 0, recs = 0, rc = FWI_OK;
-            // z-chunk rows per work item: about one item per resident CTA, so a step's
-            // critical path (one CTA streaming its chunk) stays short, but no shorter
-            // than the 2M warm-up rows each chunk streams
-            int64_t row_tiles = 0;
-            for (int si : pl.members) {
-                const fwi_request &r = reqs[slots[si].req];
-                row_tiles += (int64_t)((r.shape[2] + 2 * o.nb + 255) / 256) * (r.shape[0] + 2 * o.nb);
-            }
-            const int zchunk = (int)std::max<int64_t>(
-                2 * pl.M, std::min<int64_t>(kPoolZChunk, (row_tiles + pl.grid_step - 1) / pl.grid_step));
             h->count = 0;
             for (int si : pl.members) {
                 Slot &s = slots[si];
                 fwi::Batch2dEntry &e = h->e[h->count++];
-                rc = fwi::job_batch_entry(s.job, &e, zchunk);
+                rc = fwi::job_batch_entry(s.job, &e);
                 if (rc != FWI_OK) break;
                 e.work0 = work;
                 e.rec0 = recs;
-                work += e.xtiles * e.p.nzchunks;
+                work += e.xtiles * e.ztiles;
                 recs += e.nsamp;
                 if (!s.pool_synced) {
                     if (cudaStreamWaitEvent(pl.stream, s.turn[0], 0) != cudaSuccess) rc = FWI_ERR_CUDA;

@@ -1,6 +1,6 @@
 // Arithmetic of one 2-D step on a group of 4 points (shared by every 2-D step kernel, so
 // all of them give the same results bit for bit): the order-2M Laplacian from an x-window
-// and a z-queue, and the damped leapfrog update.
+// and z-sums, and the damped leapfrog update.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -52,17 +52,6 @@ __device__ __forceinline__ void lap_x(const float (&w)[4 + 2 * M], float4 c, con
     const float2 c0 = make_float2(cf.c0, cf.c0);
     l0 = __ffma2_rn(c0, lo2(c), __fadd2_rn(za, __fadd2_rn(make_float2(o0, om.x), ea)));
     l1 = __ffma2_rn(c0, hi2(c), __fadd2_rn(zb, __fadd2_rn(make_float2(om.y, o3), eb)));
-}
-
-// The same from a z-queue (row j + k in q[M + k]).
-template <int M>
-__device__ __forceinline__ void lap4(const float (&w)[4 + 2 * M], const float4 (&q)[2 * M + 1],
-                                     const Coefs &cf, float2 &l0, float2 &l1)
-{
-    float2 za = make_float2(0.f, 0.f), zb = za;
-#pragma unroll
-    for (int k = 1; k <= M; ++k) z_pair(cf.cz[k], q[M - k], q[M + k], za, zb);
-    lap_x<M>(w, q[M], cf, za, zb, l0, l1);
 }
 
 // The z-sums of RZ consecutive rows of a group from a column of rows in shared memory (row i

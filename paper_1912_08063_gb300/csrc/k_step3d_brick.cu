@@ -26,7 +26,9 @@
 // Brick: 32 x 8 x 8 by four warps (96^3 radius 8 18.8 / 20.4 / 25.5, 160^3 46.5 / 52.0 / 74.4),
 // 32 x 16 x 8 (19.6 / 21.0 / 28.4, 52.0 / 56.4 / 91.9), 32 x 8 x 16 (19.7 / 21.1 / 28.4, 50.7 /
 // 55.5 / 93.6) read fewer halo floats but leave fewer, larger CTAs and were no faster; one
-// plane per warp everywhere 18.7 / 20.3 / 24.3, 49.4 / 53.7 / 71.6.
+// plane per warp everywhere 18.7 / 20.3 / 24.3, 49.4 / 53.7 / 71.6.  The halo without its corners (a box
+// of the brick's columns and one for each side: 12 % fewer bytes, seven CTAs an SM instead of
+// six) was slower too: 18.4 / 22.4 / 24.5 at 96^3, 21.6 / 26.8 / 28.8 at 120^3.
 #include <cuda.h>
 #include <cuda_runtime.h>
 

@@ -29,7 +29,7 @@ struct Step3dParams {
                                   // units are numbered part-major
     int rem_first, rem_ppu;       // leftover units go to CTAs rem_first ..
                                   // rem_first + rem_ctas - 1: cut into rem_ppu aligned
-                                  // pieces each, piece-major (rem_ppu > 0), or as one run cut into
+                                  // pieces each (rem_ppu > 0), or as one run cut into
                                   // equal pieces that may cross units (rem_ppu = 0)
     float cx[kMaxM + 1], cy[kMaxM + 1], cz[kMaxM + 1], c0;
     float2 cy2[kMaxM + 1], cz2[kMaxM + 1], c02;   // the same weights as packed pairs
@@ -164,9 +164,9 @@ __host__ __device__ inline bool schedule_segment(const Step3dParams &p, int colu
     if (rem <= 0 || kk < 0 || kk >= p.rem_ctas) return false;
     const int zb = (S - 1) * p.zfirst;            // the leftover units lie in the last part
     const int len_u = p.nz - zb;
-    if (p.rem_ppu > 0) {                          // aligned pieces, one per CTA, piece-major
+    if (p.rem_ppu > 0) {                          // aligned pieces, one per CTA
         if (idx > 0) return false;
-        const int u = first + kk % rem, piece = kk / rem;
+        const int u = first + kk / p.rem_ppu, piece = kk % p.rem_ppu;
         const int plen = (len_u + p.rem_ppu - 1) / p.rem_ppu;
         *col = u % columns;
         *z0 = zb + piece * plen;
@@ -204,21 +204,25 @@ cudaError_t launch_step2d_tile(const StepParams &p, int nshots, bool img, const 
 // (each piece streams 2M warm-up planes).  A unit is a whole column, or, with `in_step`, one
 // of several z-parts of a column that begin at the same z in every column: the CTAs of a
 // round then stream z in step, so a tile's halo planes are still in L2 when its neighbours
-// read them.  Units are numbered part-major and pieces piece-major, so that tiles next to one
-// another in x run on CTAs next to one another.  With at least as many columns as CTAs,
-// columns are cut into parts where whole rounds of them leave less to the last, partial
-// round.  With fewer columns than CTAs the planner compares: the same number of parts of
-// every column, at most one to a CTA and none left over; S = ceil(resident / columns) equal
-// parts whose leftover last parts are cut over all CTAs; and S parts of which the first ones
-// are longer and the leftover last parts go to the CTAs that ran a last part.  It keeps the
-// one whose busiest CTA streams the fewest planes (warm-up planes included).
+// read them.  Units are numbered part-major, so that tiles next to one another in x run on
+// CTAs next to one another.  With at least as many columns as CTAs, columns are cut into parts
+// where whole rounds of them leave less to the last, partial round.  With fewer columns than
+// CTAs the planner compares: the same number of parts of every column, at most one to a CTA
+// and none left over; S = ceil(resident / columns) equal parts whose leftover last parts are
+// cut over all CTAs; and S parts of which the first ones are longer and the leftover last parts
+// go to the CTAs that ran a last part.  It keeps the one whose busiest CTA streams the fewest
+// planes (warm-up planes included), the first one's weighed by (resident / CTAs used)^2 at
+// radius 8: its steps are bound by the SMs' instruction issue, and idle CTAs cost more there
+// (forward at 360^3, 552 of 608 CTAs and 106 planes 162.5 us, all CTAs and 115 planes 159.3; two
+// shots of 199 x 197 x 433, 546 CTAs and 83 planes 125, all and 95 planes 122; at 296^3, 570
+// and 66 planes 97, all and 79 planes 99).
 // Every launch of the step is planned in step.  Measured on GB300 (the radius-4 reverse step
 // still with two rows per thread), us per step forward /
 // store / reverse, against one run of the columns cut over all CTAs below 96 MB and no
 // candidate without leftovers: radius 4, 216^3 39.2 / 45.5 / 69.6 -> 36.2 / 41.1 / 60.2, 280^3
 // 101 / 122 / 165 -> 63 / 72 / 109, 296^3 75.9 / 85.3 / 122 -> 70.7 / 81.5 / 122; radius 8, 240^3
 // 70 / 77 / 105 -> 55.6 / 61 / 71, 280^3 122 / 139 / 171 -> 86 / 95 / 102, 440^3 263 / 296 / 361 ->
-// 257 / 286 / 348.  Pieces numbered column by column: radius 4 360^3 122 / 152 / 214 against
+// 257 / 286 / 348.  Parts numbered column by column: radius 4 360^3 122 / 152 / 214 against
 // 119.6 / 137.8 / 212, 440^3 237 / 306 / 347 against 223 / 285 / 346.
 // Fills the schedule fields of p and returns the grid size.
 int plan_persistent(Step3dParams &p, int columns, int resident, bool in_step = false);

@@ -155,6 +155,7 @@ int plan_persistent(Step3dParams &p, int columns, int resident, bool in_step)
             best.round_ctas = best_grid = columns * best.zparts;
             best.rem_ctas = 0;
             best_cost = schedule_cost(best, columns, best_grid);
+            if (p.M == 8) best_cost = best_cost * resident * resident / ((int64_t)best_grid * best_grid);
         }
     }
     if (p.nz / S >= 4 * p.M) {

@@ -148,11 +148,18 @@ cudaError_t launch_step3d_tma(const Step3dParams &p, int mode, int ctas,
     const cudaError_t e = prepare_kernel(k);
     if (e != cudaSuccess) return e;
     if (ctas < 1) return cudaErrorInvalidValue;
-    // Programmatic launches at radius 4 (1024^3 forward call 379 -> 349 ms, 256^3 gradient 108.4
-    // -> 107.9 ms) and plain ones at radius 8, whose reverse step loses what it gains and more
-    // (512^3 gradient 375 ms plain, 395 with a programmatic reverse step, 377 and 379 with
-    // programmatic forward and storing steps).
-    if (p.M == 4) return launch_pdl(k.fn, dim3(ctas), dim3(k.threads), k.smem, s, p, mc, ma, mb, md, me);
+    // Programmatic or plain launches, whole calls on GB300.  At radius 4 programmatic ones where
+    // the launch itself shows (gradient, 100 steps: 160^3 computed points 5.22 ms against 5.34
+    // plain, 220^3 12.4 / 12.7, 250^3 16.95 / 17.03) and where columns outnumber the CTAs, so
+    // that some end a part early (1024^3 forward 348 / 375); plain ones in between, where the
+    // CTAs of the next step, waiting on an SM, slow those still at work (gradient 296^3 103.2 /
+    // 100.9, 360^3 46.9 / 46.0; forward 296^3 7.38 / 7.04, 420^3 19.5 / 19.1, 540^3 39.3 / 38.8).
+    // At radius 8 plain ones: its reverse step loses what it gains and more (512^3 gradient 375 ms
+    // plain, 395 with a programmatic reverse step, 377 and 379 with programmatic forward and
+    // storing steps).
+    const double points = (double)p.nx * p.ny * p.nz * p.nshots;
+    if (p.M == 4 && (points <= 20.0e6 || columns >= ctas))
+        return launch_pdl(k.fn, dim3(ctas), dim3(k.threads), k.smem, s, p, mc, ma, mb, md, me);
     k.fn<<<ctas, k.threads, k.smem, s>>>(p, mc, ma, mb, md, me);
     return cudaGetLastError();
 }

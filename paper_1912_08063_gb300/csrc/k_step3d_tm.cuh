@@ -715,13 +715,13 @@ k_step3d_tm(const __grid_constant__ Step3dParams p, const __grid_constant__ CUte
     }
 
     pdl_wait();
-    if (MODE != kModeAdj && blockIdx.x == 0 && c.tid == 0)
-        for (int k = 0; k < p.nshots; ++k)
-            store_bookkeeping(p.st_max, k, p.st_dtype, p.st_scale, p.err, p.max_clear);
     const int tiles_x = (p.nx + C::TX - 1) / C::TX;
     const int tiles = tiles_x * ((p.ny + C::TY - 1) / C::TY);
     s3d::walk_schedule(p, tiles * p.nshots, c.abort_flag,
                        [&](int col, int z0, int z1) { run_segment(c, col, z0, z1, tiles_x, tiles); });
+    if (MODE != kModeAdj && blockIdx.x == gridDim.x - 1 && c.tid == 0)
+        for (int k = 0; k < p.nshots; ++k)
+            store_bookkeeping(p.st_max, k, p.st_dtype, p.st_scale, p.err, p.max_clear);
     if (MODE == kModeAdj && C::GS) asm volatile("cp.async.wait_all;" ::: "memory");
     // every TMEM access of the CTA is complete before warp 0 releases the columns
     tmem_wait_st();

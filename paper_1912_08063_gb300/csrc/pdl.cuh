@@ -6,7 +6,7 @@
 // when a call starts) and then wait for the kernel before to end.  Measured on GB300, whole
 // calls: 2-D 517 x 900 at 16th order 3.09 -> 2.09 ms (500 steps), 96^3 16th-order gradient
 // 23.9 -> 20.4 ms, serving mix 39 -> 34 ms, 64-shot FWI iteration 95.9 -> 93.4 ms, 1024^3
-// forward 379 -> 349 ms.
+// forward 379 -> 349 ms.  (Which streaming steps are launched so: k_step3d.cu.)
 #pragma once
 
 #include <cuda_runtime.h>

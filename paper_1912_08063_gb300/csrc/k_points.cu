@@ -93,10 +93,10 @@ __global__ void k_point_taps(Geom g, const double *__restrict__ pos, int64_t npt
 // shuffle tree.  One thread per point walked 64 rows one after the other: 34 us for two
 // shots of 532 receivers at 3-D on GB300, now 4.9.
 template <int LANES, int ROWS>
-__global__ void __launch_bounds__(kThreads) k_sample_pts(Geom g, const float *__restrict__ f,
+__global__ void __launch_bounds__(kThreads) k_sample_pts(Geom g, const float *f,
                                                          const PointTaps *__restrict__ pts, int nshots,
-                                                         int nrec, int nt, int n, float *__restrict__ traces,
-                                                         const int *__restrict__ n_dev)
+                                                         int nrec, int nt, int n, float *traces,
+                                                         const int *n_dev)
 {
     pdl_next();
     const int64_t id = blockIdx.x * (int64_t)kThreads + threadIdx.x;
@@ -127,11 +127,11 @@ __global__ void __launch_bounds__(kThreads) k_sample_pts(Geom g, const float *__
 
 // kind 0: forward source, f += dt^2 w[s][n] wt / a+                   (q = wavelets)
 // kind 1: adjoint injection, f += factor (W / a+) wt q[s][n][r]        (q = residuals)
-__global__ void k_inject_pts(Geom g, float *__restrict__ f, const PointTaps *__restrict__ pts,
+__global__ void k_inject_pts(Geom g, float *f, const PointTaps *__restrict__ pts,
                              int npts, int per_shot, const float *__restrict__ W,
                              const float *__restrict__ sz, const float *__restrict__ sy,
-                             const float *__restrict__ sx, const float *__restrict__ q, int nt,
-                             int n, float dt2, float factor, int kind, const int *__restrict__ n_dev)
+                             const float *__restrict__ sx, const float *q, int nt,
+                             int n, float dt2, float factor, int kind, const int *n_dev)
 {
     const int rows = rows_per_point(g);
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;

@@ -95,15 +95,15 @@ k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUte
     const int plane = (int)p.g.plane;
     const int64_t off = (int64_t)zr * plane + x0;              // row zr, column x0
     const int64_t sb = (int64_t)shot * p.g.field + off;
-    float *__restrict__ prev = p.prev + sb;
+    float *prev = p.prev + sb;
     const float *__restrict__ Wp = p.W + off;
     const int afmt = p.aux_fmt;
     const int left = xin ? nz - zr : 0;                        // rows of this block in the grid
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
     float4 pv[RZ], Wv[RZ], gv[MODE == kImg ? RZ : 1];
     uint4 ur[MODE == kImg ? RZ : 1];
-    float *__restrict__ gp = MODE == kImg ? p.gacc + sb : nullptr;
-    const char *__restrict__ up =
+    float *gp = MODE == kImg ? p.gacc + sb : nullptr;
+    const char *up =
         MODE == kImg ? (const char *)p.aux + ((int64_t)shot * p.aux_stride + off) * (afmt ? 2 : 4) : nullptr;
     float sz[RZ];
 #pragma unroll
@@ -125,9 +125,9 @@ k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUte
             ur[r] = make_uint4(0u, 0u, 0u, 0u);
             if (r < left) {
                 if (afmt == 0) {
-                    ur[r] = __ldg((const uint4 *)(up + (int64_t)r * plane * 4));
+                    ur[r] = *(const uint4 *)(up + (int64_t)r * plane * 4);
                 } else {
-                    const uint2 h = __ldg((const uint2 *)(up + (int64_t)r * plane * 2));
+                    const uint2 h = *(const uint2 *)(up + (int64_t)r * plane * 2);
                     ur[r].x = h.x;
                     ur[r].y = h.y;
                 }

@@ -35,6 +35,8 @@
 // 95.0 / 114.2.  Larger CTAs (4 x 2, 8 x 2, 8 x 4) were slower than 2 x 2 in an earlier form.
 #include <cuda.h>
 
+#include <algorithm>
+
 #include "code16.cuh"
 #include "fwi_internal.h"
 #include "k_step3d.cuh"
@@ -69,15 +71,16 @@ __device__ __forceinline__ void tma_tile(void *dst, const CUtensorMap *map, int 
         : "memory");
 }
 
-// Warps and CTAs per SM, and rows per thread of each mode (see above).
+// Warps and CTAs per SM, and rows per thread of each mode (see above); tile rows a launch holds.
 constexpr int kWarps = 2, kMinCtas = 8;
+constexpr int kGridYMax = 65535;
 __host__ __device__ constexpr int tile_rz(int mode) { return mode == kImg ? 3 : 4; }
 
 // TAPS: an off-grid source is added too (an instantiation of its own, so that the common one
 // pays nothing for it: 3 % of a 64-shot step).
 template <int M, int MODE, bool TAPS>
 __global__ void __launch_bounds__(32 * kWarps, kMinCtas)
-k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUtensorMap map)
+k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUtensorMap map, int row0)
 {
     constexpr int RZ = tile_rz(MODE), TZ = kWarps * RZ, SX = kTileX + 2 * M, SZ = TZ + 2 * M;
     __shared__ __align__(128) float tile[SZ][SX];
@@ -90,7 +93,8 @@ k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUte
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    const int x0 = blockIdx.x * kTileX + 4 * lane, zr = blockIdx.y * TZ + warp * RZ;
+    const int tz = row0 + blockIdx.y;                           // tile row
+    const int x0 = blockIdx.x * kTileX + 4 * lane, zr = tz * TZ + warp * RZ;
     const bool xin = x0 < nx;
     const int plane = (int)p.g.plane;
     const int64_t off = (int64_t)zr * plane + x0;              // row zr, column x0
@@ -115,7 +119,7 @@ k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUte
     pdl_wait();
     if (threadIdx.x == 0) {
         mbar_expect_tx(&bar, SX * SZ * 4);
-        tma_tile(&tile[0][0], &map, blockIdx.x * kTileX - M, blockIdx.y * TZ - M, shot, &bar);
+        tma_tile(&tile[0][0], &map, blockIdx.x * kTileX - M, tz * TZ - M, shot, &bar);
     }
 #pragma unroll
     for (int r = 0; r < RZ; ++r) {
@@ -165,7 +169,7 @@ k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUte
         }
     }
     const float ainv = (MODE == kImg && p.aux_scale) ? 1.0f / p.aux_scale[2 * shot] : 1.0f;
-    if (MODE != kImg && threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0)
+    if (MODE != kImg && threadIdx.x == 0 && blockIdx.x == 0 && tz == 0)
         store_bookkeeping(p.st_max, shot, p.st_dtype, p.st_scale, p.err, p.max_clear);
     __syncthreads();   // the barrier is initialised
     const bool ok = mbar_wait(&bar, 0);
@@ -259,10 +263,15 @@ template <int M, int MODE>
 cudaError_t go(const StepParams &p, int nshots, const CUtensorMap &map, cudaStream_t s)
 {
     constexpr int TZ = kWarps * tile_rz(MODE);
-    const dim3 grid((p.g.nx + kTileX - 1) / kTileX, (p.g.nz + TZ - 1) / TZ, nshots);
-    if (MODE != kImg && p.src_pts)
-        return launch_pdl(k_step2d_tile<M, MODE, MODE != kImg>, grid, dim3(32 * kWarps), 0, s, p, map);
-    return launch_pdl(k_step2d_tile<M, MODE, false>, grid, dim3(32 * kWarps), 0, s, p, map);
+    auto *fn = MODE != kImg && p.src_pts ? k_step2d_tile<M, MODE, MODE != kImg> : k_step2d_tile<M, MODE, false>;
+    // tile rows on grid.y, at most 65535 a launch (a launch writes its own rows of prev only)
+    const int rows = (p.g.nz + TZ - 1) / TZ;
+    cudaError_t e = cudaSuccess;
+    for (int row0 = 0; row0 < rows && e == cudaSuccess; row0 += kGridYMax) {
+        const dim3 grid((p.g.nx + kTileX - 1) / kTileX, std::min(rows - row0, kGridYMax), nshots);
+        e = launch_pdl(fn, grid, dim3(32 * kWarps), 0, s, p, map, row0);
+    }
+    return e;
 }
 
 }  // namespace

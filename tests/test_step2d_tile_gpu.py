@@ -56,3 +56,32 @@ def test_tile_step_matches_oracle(order, nz, nx, nb, nshots, snap, monkeypatch):
     e = (_rel(tr, ref), _rel(fin.reshape(rfin.shape), rfin), _rel(g, np.asarray(rg).reshape(g.shape)))
     print(f"tile {nz}x{nx} nb {nb} o{order} {snap}: traces {e[0]:.1e} final {e[1]:.1e} grad {e[2]:.1e}")
     assert e[0] <= 1e-4 and e[1] <= 1e-4 and e[2] <= (1e-3 if snap == "fp32" else 1e-2)
+
+
+@pytest.mark.parametrize("order,lo,hi,row", [
+    (8, 523984, 524384, 524268),    # tile rows beyond 65535 of 8 rows: forward modes
+    (16, 523984, 524384, 524276),
+    (8, 393000, 393400, 393200),    # beyond 65535 of 6 rows: the reverse step
+])
+def test_more_tile_rows_than_a_launch_holds(order, lo, hi, row):
+    """A grid of 524,400 computed rows: the rows around the last tile of a launch equal those of a
+    model of rows lo .. hi - 1 alone, whose faces the waves do not reach (12 steps carry them at
+    most 96 rows), bit for bit."""
+    from paper_1912_08063_gb300 import fwi
+    nz, nx, nb, nt, h = 524384, 12, 8, 12, 10.0
+    dt = 0.3 * h / 4600.0
+    v = np.random.default_rng(order).uniform(1600.0, 4400.0, (nz, nx)).astype(np.float32)
+    wav = torch.from_numpy(synth.ricker(120.0, dt, nt)[None].astype(np.float32)).cuda()
+    outs = []
+    for a, b in ((0, nz), (lo, hi)):
+        m = fwi.FwiModel(torch.from_numpy(v[a:b]).cuda(), h, dt, nt, order=order, nb=nb, sponge_vref=4600.0)
+        src = np.array([[row - a, 0, nx // 2]], dtype=np.int32)
+        rec = np.array([[row - a + 8, 0, x] for x in range(nx)], dtype=np.int32)
+        acq = fwi.Acquisition(src, rec)
+        tr, fin = m.forward(acq, wav, final_state=True)
+        phi, g = m.gradient(acq, wav, tr * 0.5)
+        fin = fin.reshape(-1, nx + 2 * nb)[nb + lo - a:nb + hi - a]
+        outs.append([x.cpu().numpy() for x in (tr, fin, phi, g[lo - a:hi - a])])
+        m.close()
+    for x, y in zip(*outs):
+        assert np.abs(x).max() > 0 and np.array_equal(x, y)

@@ -41,12 +41,16 @@ int fwi::report_error(int code, const std::string &msg) { return fail(code, msg)
 
 namespace {
 
+// Returns a failed call's error, and takes it from the runtime: what is left there would be
+// reported by the next kernel launch that asks for its own.
 #define FWI_CU(call)                                                                     \
     do {                                                                                 \
         cudaError_t e_ = (call);                                                         \
-        if (e_ != cudaSuccess)                                                           \
+        if (e_ != cudaSuccess) {                                                         \
+            cudaGetLastError();                                                          \
             return fail(e_ == cudaErrorMemoryAllocation ? FWI_ERR_OOM : FWI_ERR_CUDA,    \
                         std::string(#call) + ": " + cudaGetErrorString(e_));             \
+        }                                                                                \
     } while (0)
 
 #define FWI_TRY(expr)             \

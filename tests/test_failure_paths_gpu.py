@@ -1,5 +1,5 @@
 """Failure paths reached on purpose without a GPU fault: a bounded device wait that runs
-out (FWI_ERR_TIMEOUT, latched per model) and a memory budget too small for a request
+out (FWI_ERR_TIMEOUT, latched per model), a launch that the runtime refuses, and a memory budget too small for a request
 (FWI_ERR_OOM before anything is launched for it)."""
 import math
 
@@ -40,6 +40,23 @@ def test_bounded_wait_runs_out_and_latches_timeout():
     fwi.fwi_sync_status(m2.handle)
     m2.close()
     assert np.array_equal(before, after)
+
+
+def test_refused_launch_fails_its_own_call_only():
+    """65,536 shots exceed a launch grid's third extent, which the runtime refuses before anything
+    runs; the calls after it are not told of that error."""
+    from paper_1912_08063_gb300 import fwi
+    shots, nt = 65536, 4
+    m = fwi.FwiModel(np.full((8, 8), 2000.0, np.float32), 10.0, 1e-3, nt, nb=0)
+    acq = fwi.Acquisition(np.full((shots, 3), [3, 0, 3], np.int32), np.array([[4, 0, 2]], np.int32))
+    with pytest.raises(fwi.FwiError) as e:
+        m.forward(acq, torch.zeros(shots, nt, device="cuda"))
+    assert e.value.code == fwi.FWI_ERR_CUDA
+    m.close()
+    w, m = _small_model(fwi, np.random.default_rng(23))
+    tr = m.forward(fwi.Acquisition(w.src, w.rec), torch.from_numpy(w.wavelets()).cuda())
+    assert torch.isfinite(tr).all() and tr.abs().max() > 0
+    m.close()
 
 
 def test_selftest_rejects_poll_limits_out_of_range():

@@ -461,15 +461,26 @@ void brick_boxes(int M, int (&mid)[3], int (&arm)[3])
     arm[0] = C::TX, arm[1] = C::TY, arm[2] = M;
 }
 
+// Bricks lie on a grid of x, y and z times shots, whose last two extents end at 65535.  Thin grids of
+// many planes, rows or shots that exceed them stream (a one-dimensional grid).
+static bool brick_grid_fits(const Step3dParams &p)
+{
+    using C = Brick<4, kModeStep, true>;   // the brick's extents are the same in every form
+    const int64_t ty = (p.ny + C::TY - 1) / C::TY, tz = (p.nz + C::TZ - 1) / C::TZ;
+    return ty <= 65535 && tz * p.nshots <= 65535;
+}
+
 // Whether a launch takes bricks: up to the points of all shots below which they measured
 // faster than streaming (us, bricks / streaming).  Radius 4: forward 20.9 / 22.8 at 176^3
 // computed points and 24.9 / 24.9 at 184^3, store 24.4 / 25.3 at 168^3 and 26.9 / 26.1 at 176^3,
 // reverse 20.2 / 22.4 at 136^3, 22.2 / 22.3 at 144^3 and 24.9 / 24.5 at 152^3.  Radius 8: forward
 // 34.1 / 34.8 at 192^3 and 47.6 / 47.3 at 208^3, store 30.7 / 32.9 at 168^3 and 34.5 / 33.7 at
-// 176^3, reverse 27.4 / 32.3 at 160^3 and 40.2 / 36.7 at 168^3.  FWI_STEP3D_BRICK=0/1 overrides;
+// 176^3, reverse 27.4 / 32.3 at 160^3 and 40.2 / 36.7 at 168^3.  FWI_STEP3D_BRICK=0/1 overrides (1
+// where the grid fits);
 // the switches that choose among the streaming kernels turn bricks off.
 bool step3d_use_brick(const Step3dParams &p, int mode)
 {
+    if (!brick_grid_fits(p)) return false;
     if (const char *e = std::getenv("FWI_STEP3D_BRICK")) return std::atoi(e) != 0;
     for (const char *v : {"FWI_STEP3D_TMEM", "FWI_STEP3D_VARIANT", "FWI_STEP3D_HALF", "FWI_STEP3D_TILE_G"})
         if (std::getenv(v)) return false;

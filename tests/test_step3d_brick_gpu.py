@@ -51,3 +51,30 @@ def test_brick_equals_streaming(order, shape, nb, h, nshots, snap, slots, monkey
         for a, b in zip(outs[0], other):
             assert np.array_equal(a, b)
     assert np.isfinite(outs[0][3]).all() and np.abs(outs[0][3]).max() > 0
+
+
+@pytest.mark.parametrize("shape,shots,grad", [
+    ((262200, 4, 4), 1, True),      # 65550 bricks in z
+    ((4, 524320, 2), 1, True),      # 65540 in y
+    ((4, 4, 4), 65600, False),      # one in z for each shot
+])
+def test_thin_grids_beyond_a_launch_grid_stream(shape, shots, grad, monkeypatch):
+    """Few points, but more bricks along an axis than a launch grid takes: the streaming kernels
+    run the call, as they do with bricks off."""
+    from paper_1912_08063_gb300 import fwi
+    nt, dt = 10, 0.3 * 10.0 / 4600.0
+    v = torch.from_numpy(np.random.default_rng(5).uniform(1600.0, 4400.0, shape).astype(np.float32)).cuda()
+    src = np.broadcast_to(np.array(shape) // 2, (shots, 3)).astype(np.int32)
+    rec = src[:1] + np.array([[1, 0, 0]], np.int32)
+    wav = torch.from_numpy(np.tile(synth.ricker(120.0, dt, nt), (shots, 1)).astype(np.float32)).cuda()
+    outs = []
+    for brick in (None, "0"):
+        if brick:
+            monkeypatch.setenv("FWI_STEP3D_BRICK", brick)
+        m = fwi.FwiModel(v, 10.0, dt, nt, order=16, nb=0, sponge_vref=4600.0)
+        acq = fwi.Acquisition(src, rec)
+        tr = m.forward(acq, wav)
+        outs.append([tr, *(m.gradient(acq, wav, tr * 0.5) if grad else ())])
+        m.close()
+    for a, b in zip(*outs):
+        assert a.abs().max() > 0 and torch.equal(a, b)

@@ -115,9 +115,17 @@ bool is_device_ptr(const void *p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Device memory that its owner frees by going away.
 struct DevBuf {
     void *p = nullptr;
     size_t bytes = 0;
+    DevBuf() = default;
+    DevBuf(const DevBuf &) = delete;
+    DevBuf &operator=(const DevBuf &) = delete;
+    ~DevBuf()
+    {
+        if (p) cudaFree(p);
+    }
     int ensure(size_t want)
     {
         if (want <= bytes && p) return FWI_OK;
@@ -133,12 +141,6 @@ struct DevBuf {
         }
         bytes = want;
         return FWI_OK;
-    }
-    void release()
-    {
-        if (p) cudaFree(p);
-        p = nullptr;
-        bytes = 0;
     }
     template <class T> T *as() const { return (T *)p; }
 };
@@ -227,7 +229,8 @@ struct fwi_model {
     {
         size_t b = v.bytes + W.bytes + sig.bytes + g32.bytes + g64.bytes + traces.bytes +
                    src_off.bytes + rec_off.bytes + inj.bytes + src_scale.bytes + maxbits.bytes +
-                   partials.bytes + phi.bytes + snaps.bytes + scales.bytes + rec_map.bytes;
+                   partials.bytes + phi.bytes + snaps.bytes + scales.bytes + rec_map.bytes +
+                   src_pts.bytes + rec_pts.bytes + step_ctr.bytes + cl_desc.bytes + cl_off.bytes;
         for (int i = 0; i < 2; ++i) b += u[i].bytes + mu[i].bytes + stage_out[i].bytes;
         for (int i = 0; i < 3; ++i) b += stage_in[i].bytes;
         return (int64_t)b;
@@ -2194,31 +2197,7 @@ void fwi_destroy(fwi_model *m)
 {
     if (!m) return;
     if (m->last_stream) cudaStreamSynchronize(m->last_stream);
-    m->v.release();
-    m->W.release();
-    m->sig.release();
-    for (int i = 0; i < 2; ++i) {
-        m->u[i].release();
-        m->mu[i].release();
-        m->stage_out[i].release();
-    }
-    for (int i = 0; i < 3; ++i) m->stage_in[i].release();
-    m->g32.release();
-    m->g64.release();
-    m->traces.release();
-    m->src_off.release();
-    m->rec_off.release();
-    m->inj.release();
-    m->src_scale.release();
-    m->maxbits.release();
-    m->partials.release();
-    m->phi.release();
-    m->snaps.release();
-    m->scales.release();
     if (m->h_flag) cudaFreeHost(m->h_flag);
-    m->cl_desc.release();
-    m->cl_off.release();
-    m->rec_map.release();
     for (cudaEvent_t e : m->ev) cudaEventDestroy(e);
     delete m;
 }

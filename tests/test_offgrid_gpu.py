@@ -118,3 +118,34 @@ def test_offgrid_point_outside_is_rejected():
                           rec_pos=np.array([[[5.0, 0.0, 5.0]]]))   # taps cross the grid edge
     with pytest.raises(RuntimeError):
         m.forward(bad, wav)
+
+
+def _run_many_points(offgrid):
+    """device_bytes of a model after a forward call with 32,768 receivers; the model is closed."""
+    from paper_1912_08063_gb300 import fwi
+    rng = np.random.default_rng(77)
+    nt, shots, nrec = 4, 64, 512
+    src = np.stack([np.full(shots, 5.0), np.zeros(shots), np.linspace(2, 57, shots)], 1)
+    rec = np.stack([rng.uniform(0, 39, (shots, nrec)), np.zeros((shots, nrec)), rng.uniform(0, 59, (shots, nrec))], 2)
+    acq = (fwi.Acquisition(src_pos=src, rec_pos=rec) if offgrid
+           else fwi.Acquisition(src.astype(np.int32), rec.astype(np.int32)))
+    m = fwi.FwiModel(torch.full((40, 60), 2000.0).cuda(), 10.0, 1e-3, nt)
+    m.forward(acq, torch.zeros(shots, nt).cuda())
+    n = m.info()["device_bytes"]
+    m.close()
+    return n
+
+
+def test_tap_tables_are_in_device_bytes():
+    assert _run_many_points(True) >= _run_many_points(False) + 112 * 64 * 512   # 112 bytes a point
+
+
+def test_models_with_offgrid_points_return_their_memory():
+    """Eight models one after another leave the free memory where the first left it."""
+    _run_many_points(True)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    for _ in range(8):
+        _run_many_points(True)
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] < 8 << 20     # a table is 3.7 MB

@@ -67,7 +67,10 @@ typedef struct {
                                    velocity of the model at creation                     */
     int32_t timing;             /* 1: bracket every time-step launch with CUDA events and
                                    accumulate kernel times (read with fwi_model_info);
-                                   the call then waits for its stream at the end        */
+                                   the call then waits for its stream at the end.  Steps
+                                   are then launched one by one and do not overlap, so
+                                   2-D calls that would run on chip (below) are timed in
+                                   single steps                                          */
     int32_t temporal_blocking;  /* 0 (default) and 2: 2-D calls on grids whose states fit in
                                    the shared memory of one cluster of CTAs per shot, with
                                    node sources and node receivers on one row, advance many
@@ -252,8 +255,9 @@ int fwi_model_info(const fwi_model *m, fwi_info *out);
  * as they have arrived, a slot is free and their device-memory estimate fits in the
  * budget's remainder; an admitted request owns a model (wavefields and checkpoints stay
  * on the device) and a stream, and one host thread issues the admitted requests' time
- * steps round-robin (steps_per_turn at a time, at most two turns in flight per request),
- * so their work overlaps on the device.  2-D forward requests with node source and
+ * steps round-robin (steps_per_turn at a time, at most two turns in flight per request;
+ * a request that steps on chip 64 or more at a time, one turn in flight), so their work
+ * overlaps on the device.  2-D forward requests with node source and
  * receivers share one launch instead: each tick, one captured graph of persistent
  * multi-request step and sampling kernels advances all of them by steps_per_turn
  * (rounded up to even) steps from a device table of request descriptors updated in
@@ -299,7 +303,8 @@ typedef struct {
 typedef struct {
     int64_t hbm_budget_bytes;   /* device memory for admitted requests (0: 80 % free)   */
     int32_t max_active;         /* admitted requests at once (default 16)               */
-    int32_t steps_per_turn;     /* time steps issued per request per turn (default 8)   */
+    int32_t steps_per_turn;     /* time steps issued per request per turn (default 8); a
+                                   request that steps on chip issues 64 or more          */
     int32_t snap_slots;         /* checkpoint budget per gradient request, in pairs
                                    (default 64; slots holding u^n alone take half)      */
     int32_t nb;                 /* sponge width (default 20)                            */

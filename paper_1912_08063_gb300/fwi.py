@@ -359,7 +359,11 @@ class Acquisition:
 
 
 class FwiModel:
-    """A velocity model on the device with its numerics; methods mirror the C ABI."""
+    """A velocity model on the device with its numerics; methods mirror the C ABI.
+
+    temporal_blocking takes the values of fwi_opts (0: many steps per launch on chip where a
+    2-D grid fits; 1: single steps only; 2: as 0) or a bool: True asks for blocking (2),
+    False for the default."""
 
     def __init__(self, v, spacing, dt, nt, order=8, nb=20, snap_dtype="fp32",
                  snap_budget_bytes=0, sponge_r0=1e-3, sponge_vref=0.0, fold_every=256,
@@ -382,7 +386,7 @@ class FwiModel:
         self.opts = fwi_opts(int(order), int(nb) if nb else -1, SNAP_DTYPES[snap_dtype],
                              int(fold_every), int(snap_budget_bytes), float(sponge_r0),
                              float(sponge_vref), int(bool(timing)),
-                             int(temporal_blocking))
+                             2 if temporal_blocking is True else int(temporal_blocking))
         self.handle = fwi_create_model(self.ndim, self.shape, sp, v, dt, nt, self.opts,
                                        stream)
 

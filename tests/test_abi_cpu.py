@@ -189,3 +189,12 @@ def test_host_functions_reject_bad_arguments():
         assert e.value.code == fwi.FWI_ERR_ARG
     assert fwi.fwi_cfl_number(4, 8, (10.0, 10.0, 10.0), 3000.0, 1e-3) < 0      # bad ndim
     assert fwi.fwi_cfl_number(3, 9, (10.0, 10.0, 10.0), 3000.0, 1e-3) < 0      # odd order
+
+
+@pytest.mark.parametrize("asked,value", [(True, 2), (False, 0), (0, 0), (1, 1), (2, 2)])
+def test_temporal_blocking_true_asks_for_blocking(asked, value, monkeypatch):
+    """The option's value 1 means single steps only; True must not become it."""
+    seen = []
+    monkeypatch.setattr(fwi, "fwi_create_model", lambda *a: seen.append(a[6].temporal_blocking))
+    fwi.FwiModel(np.full((8, 8), 2000.0, np.float32), 10.0, 1e-3, 4, temporal_blocking=asked)
+    assert seen == [value]

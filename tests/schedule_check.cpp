@@ -1,14 +1,25 @@
 // Host-side check of the persistent 3-D step schedule, built from the library's own
 // sources: plan_persistent (tmap.cpp) fills a launch's schedule, schedule_segment
 // (step3d.h) enumerates what each CTA streams, and every (tile column, output plane) must
-// be computed exactly once.  Prints "ok <combinations>" or the first failure.
+// be computed exactly once.  Prints "ok <combinations>" or the first failure.  With the
+// arguments M nz columns resident it prints that launch's plan instead: "rounds zparts rem_ctas
+// rem_first rem_ppu".
 #include <cstdio>
+#include <cstdlib>
 #include <vector>
 
 #include "step3d.h"
 
-int main()
+int main(int argc, char **argv)
 {
+    if (argc == 5) {
+        fwi::Step3dParams p{};
+        p.M = std::atoi(argv[1]);
+        p.nz = std::atoi(argv[2]);
+        fwi::plan_persistent(p, std::atoi(argv[3]), std::atoi(argv[4]), true);
+        std::printf("%d %d %d %d %d\n", p.rounds, p.zparts, p.rem_ctas, p.rem_first, p.rem_ppu);
+        return 0;
+    }
     const int nzs[] = {20, 33, 64, 100, 296, 440, 552, 1000};
     const int Ms[] = {4, 8};
     const int colss[] = {1, 2, 3, 50, 95, 151, 152, 153, 162, 200, 303, 304, 305, 315, 607,

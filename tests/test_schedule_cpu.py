@@ -14,7 +14,8 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
 
 
-def test_persistent_schedule_covers_every_unit_once(tmp_path):
+def build_check(tmp_path):
+    """Builds schedule_check.cpp; returns a function that runs it with arguments."""
     cxx = shutil.which("g++")
     if cxx is None or not os.path.exists(os.path.join(CUDA, "include", "cuda_runtime.h")):
         pytest.skip("g++ and the CUDA headers are needed to build the check")
@@ -26,7 +27,16 @@ def test_persistent_schedule_covers_every_unit_once(tmp_path):
     r = subprocess.run(cmd, capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
     env = dict(os.environ, LD_LIBRARY_PATH=f"{CUDA}/lib64:" + os.environ.get("LD_LIBRARY_PATH", ""))
-    out = subprocess.run([exe], capture_output=True, text=True, env=env, timeout=120)
-    assert out.returncode == 0, out.stdout + out.stderr
-    assert out.stdout.startswith("ok "), out.stdout
-    assert int(out.stdout.split()[1]) == 8 * 2 * 18 * 6 * 2
+
+    def run(*args):
+        out = subprocess.run([exe, *map(str, args)], capture_output=True, text=True, env=env, timeout=120)
+        assert out.returncode == 0, out.stdout + out.stderr
+        return out.stdout
+
+    return run
+
+
+def test_persistent_schedule_covers_every_unit_once(tmp_path):
+    out = build_check(tmp_path)()
+    assert out.startswith("ok "), out
+    assert int(out.split()[1]) == 8 * 2 * 18 * 6 * 2

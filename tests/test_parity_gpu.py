@@ -502,11 +502,10 @@ def test_gradient_from_host_buffers():
         assert rel(g_h, rg) <= TOL_GRAD16 and abs(phi_h[0] - rphi) <= TOL_GRAD32 * rphi
 
 
-def test_2d_batch_with_l2_prefetch_equals_single_shots():
-    """A 2-D batch whose fields exceed 96 MB (64 shots of the faulted model, 440 x 1064
-    computed points, 120 MB per field) runs its steps with the streamed rows prefetched
-    into L2; one-shot calls of the same shots run without.  The prefetches change no
-    arithmetic: the traces equal bit for bit, and the batch's FP64 gradient equals the sum
+def test_2d_batch_equals_single_shots():
+    """A 2-D batch whose two states exceed the L2 (64 shots of the faulted model, 440 x 1064
+    computed points, 120 MB per field) against one-shot calls of the same shots, whose states
+    stay in it: the traces equal bit for bit, and the batch's FP64 gradient equals the sum
     of the one-shot FP64 gradients to rounding."""
     f = fwi()
     w = synth.faulted_2d(nt=120)
@@ -529,12 +528,8 @@ def test_2d_batch_with_l2_prefetch_equals_single_shots():
     m.close()
 
 
-@pytest.mark.parametrize("tma", ["1", "0"])
-def test_2d_step_kernels_both_variants(tma, monkeypatch):
-    """The 2-D step runs either the register-streaming kernel (default) or the TMA-staged
-    one (FWI_STEP2D_TMA=1); traces and FP32-checkpoint gradients equal each other bit for
-    bit and match the oracle, for a batch of shots at orders 8 and 16."""
-    monkeypatch.setenv("FWI_STEP2D_TMA", tma)
+def test_2d_steps_match_oracle_at_both_orders():
+    """Traces and FP32-checkpoint gradients of the 2-D steps at orders 8 and 16 match the oracle."""
     rng = np.random.default_rng(33)
     for order in (8, 16):
         w = synth.random_small(rng, 2, (61, 300), nt=90, order=order, nb=6, nrec=11)
@@ -546,7 +541,7 @@ def test_2d_step_kernels_both_variants(tma, monkeypatch):
         phi, g = m.gradient(acq, wav, torch.from_numpy(dobs).cuda())
         rphi, rg = p.gradient(dobs.astype(np.float64))
         et, eg = rel(tr, ref), rel(g.cpu().numpy(), rg)
-        print(f"2-D order {order}, TMA {tma}: traces {et:.2e}, gradient {eg:.2e}")
+        print(f"2-D order {order}: traces {et:.2e}, gradient {eg:.2e}")
         assert et <= TOL_FWD and eg <= TOL_GRAD32
 
 

@@ -1,9 +1,7 @@
-"""Temporal blocking of the 2-D forward step (fwi_opts.temporal_blocking).  Mode 1: a batch
-of shots wide enough to fill the GPU advances two time steps per pass; its traces and final
-state equal the single-step path (each shot on its own, too few shots for the two-step
-pass) bit for bit, including an odd step count (the last step single), and match the FP64
-oracle.  Mode 2: a one-shot request small enough for one cluster of CTAs advances up to 64
-steps per launch with its states in shared memory; the same bars."""
+"""2-D stepping on chip (fwi_opts.temporal_blocking) against single steps and the oracle.  A
+batch of more shots than clusters of CTAs run at once goes step by step, its shots one at a time
+go on chip, many steps per launch with the states in shared memory: traces and final states are
+equal bit for bit, for odd step counts too."""
 import numpy as np
 import pytest
 
@@ -29,21 +27,24 @@ def _case(order, nshots, nt, seed):
 
 
 @pytest.mark.parametrize("order,nshots,nt", [(8, 48, 61), (16, 80, 40)])
-def test_two_step_pass_equals_single_steps(order, nshots, nt):
+def test_batch_in_single_steps_equals_shots_on_chip(order, nshots, nt):
     from paper_1912_08063_gb300 import fwi
     v, h, dt, src, rec, wav = _case(order, nshots, nt, seed=order)
     m = fwi.FwiModel(torch.from_numpy(v).cuda(), h, dt, nt, order=order, sponge_vref=4600.0,
                      temporal_blocking=True)
     tr, fin = m.forward(fwi.Acquisition(src, rec), torch.from_numpy(wav).cuda(), final_state=True)
     tr, fin = tr.cpu().numpy(), fin.cpu().numpy()
+    launches = m.info()["kernel_launches"]
+    assert launches >= nt                       # a launch or more per step
     for s in (0, nshots // 2, nshots - 1):
         t1, f1 = m.forward(fwi.Acquisition(src[s:s + 1], rec), torch.from_numpy(wav[s:s + 1]).cuda(),
                            final_state=True)
         assert np.array_equal(tr[s], t1.cpu().numpy()[0])
         assert np.array_equal(fin[s], f1.cpu().numpy()[0])
+    assert m.info()["kernel_launches"] - launches < nt   # three calls of a few launches
 
 
-def test_two_step_pass_matches_oracle():
+def test_batch_of_shots_matches_oracle():
     from paper_1912_08063_gb300 import fwi
     nshots, nt = 48, 50
     v, h, dt, src, rec, wav = _case(8, nshots, nt, seed=3)
@@ -55,16 +56,15 @@ def test_two_step_pass_matches_oracle():
                        wavelet=wav[pick].astype(np.float64))
     ref = P.forward()
     e = np.linalg.norm(tr[pick] - ref) / np.linalg.norm(ref)
-    print(f"two-step pass traces vs oracle: rel-L2 {e:.2e}")
+    print(f"batch traces vs oracle: rel-L2 {e:.2e}")
     assert e <= 1e-4
 
 
 @pytest.mark.parametrize("shape,order", [((60, 90), 8), ((131, 77), 16), ((300, 280), 8)])
 def test_onchip_blocking_equals_single_steps(shape, order):
-    """temporal_blocking = 2: a one-shot 2-D forward with receivers on one row runs up to
-    64 steps per launch in one cluster of CTAs with both states in shared memory; traces
-    and the final state equal single steps bit for bit, and the traces match the
-    oracle."""
+    """temporal_blocking 0 and 2 run a one-shot 2-D forward with receivers on one row on chip:
+    traces and the final state equal those of single steps (1) bit for bit, in fewer launches,
+    and the traces match the oracle."""
     from paper_1912_08063_gb300 import fwi
     import oracle
     rng = np.random.default_rng(41)
@@ -76,14 +76,17 @@ def test_onchip_blocking_equals_single_steps(shape, order):
     rec = np.array([[2, 0, x] for x in range(nx)], dtype=np.int32)
     wav = synth.ricker(25.0, dt, nt)[None].astype(np.float32)
     acq = fwi.Acquisition(src, rec)
-    outs = []
-    for tb in (0, 2):
+    outs, launches = [], []
+    for tb in (1, 0, 2):
         m = fwi.FwiModel(torch.from_numpy(v).cuda(), h, dt, nt, order=order, nb=20,
                          temporal_blocking=tb)
         tr, fin = m.forward(acq, torch.from_numpy(wav).cuda(), final_state=True)
         outs.append((tr.cpu().numpy(), fin.cpu().numpy()))
+        launches.append(m.info()["kernel_launches"])
         m.close()
-    assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
+    for other in outs[1:]:
+        assert np.array_equal(outs[0][0], other[0]) and np.array_equal(outs[0][1], other[1])
+    assert launches[1] == launches[2] < nt <= launches[0]
     ref = oracle.Problem(v, h, dt, nt, order=order, nb=20, src=src, rec=rec,
                          wavelet=wav).forward()
     e = np.linalg.norm(outs[1][0] - ref) / np.linalg.norm(ref)

@@ -14,7 +14,7 @@ namespace fwi {
 
 // Configuration per radius and mode; FWI_STEP3D_VARIANT=<ty>,<ry>,<pf>,<u>,<opt>[,<opt_rev>]
 // overrides the register-queue kernel's configuration for tuning runs (only the
-// instantiated combinations are accepted), and FWI_STEP3D_TMEM=0/1 turns the
+// instantiated combinations are accepted; radius 4's reverse mode has one form), and FWI_STEP3D_TMEM=0/1 turns the
 // tensor-memory kernel off/on in every mode, and FWI_STEP3D_TILE_G=0/1 fixes the form of
 // its reverse step (g staged per thread / g as a TMA tile; unset: by the launch's CTAs
 // per tile column, kTileGParts).  By default, as measured on GB300: the

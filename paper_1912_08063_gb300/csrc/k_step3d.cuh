@@ -733,11 +733,10 @@ Step3dKernelInfo adj_info()
     return k;
 }
 
-// The same in `mode`.
+// The same in forward mode `mode`.
 template <int M, int TY, int RY, int P, int U, int F>
-Step3dKernelInfo kernel_info(int mode)
+Step3dKernelInfo fwd_info(int mode)
 {
-    if (mode == kModeAdj) return adj_info<M, TY, RY, P, U, F>();
     Step3dKernelInfo k;
     using C = Cfg<M, TY, RY, P, U, F, 2>;
     k.fn = mode == kModeStep ? (Step3dKernel)k_step3d_tma<M, TY, RY, P, U, F, kModeStep>
@@ -745,6 +744,12 @@ Step3dKernelInfo kernel_info(int mode)
     k.threads = C::NT;
     k.smem = C::SMEM;
     return k;
+}
+
+template <int M, int TY, int RY, int P, int U, int F>
+Step3dKernelInfo kernel_info(int mode)
+{
+    return mode == kModeAdj ? adj_info<M, TY, RY, P, U, F>() : fwd_info<M, TY, RY, P, U, F>(mode);
 }
 
 }  // namespace s3d

@@ -528,8 +528,9 @@ __global__ void k_fold(float *__restrict__ g32, double *__restrict__ g64, int64_
     }
 }
 
-// 1 / v for FP32 v as the sum of three FP32 terms: each residual 1 - v (sum so far) is exact
-// in one FMA, so the terms leave a relative error below 2^-68, under FP64's rounding.  v
+// 1 / v for FP32 v as the sum of three FP32 terms, each from the residual 1 - v (sum so far)
+// that one FMA gives (the first exactly, the second to FP32): the terms leave a relative error
+// below 2^-68, under FP64's rounding.  v
 // outside 2^-60 .. 2^60 takes the FP64 division (its residuals could underflow).
 __device__ __forceinline__ double recip(float v)
 {

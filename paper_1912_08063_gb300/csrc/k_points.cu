@@ -1,6 +1,6 @@
 // Off-grid sources and receivers: sampling, injection and the point terms of the
-// transposed imaging sum for points given as Kaiser-windowed sinc taps (the tap tables
-// are built on the host, api.cpp).  A point's taps are the nodes (z0 + a, y0 + b, x0 + c),
+// transposed imaging sum for points given as Kaiser-windowed sinc taps (k_point_taps builds
+// the tap tables from the positions).  A point's taps are the nodes (z0 + a, y0 + b, x0 + c),
 // a, c < 8 and b < ty (8 in 3-D, 1 in 2-D), with weight wz[a] wy[b] wx[c].  Sampling
 // sums the weighted taps; every injection spreads a value over the same taps with the
 // same weights, so injection is the exact transpose of sampling.  One thread handles one

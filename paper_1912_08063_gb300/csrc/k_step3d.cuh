@@ -120,8 +120,8 @@ __device__ __forceinline__ void tma_prefetch4(const CUtensorMap *map, int x, int
 __device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
 
-// Approximate reciprocal (PTX rcp.approx), the operation behind the fast division it
-// replaces; the damping factor 1 + s lies in [1, 2).
+// Approximate reciprocal of the damping factor 1 + s, a normal number near 1: rcp.approx.ftz is
+// within 1 ulp of the exact one (PTX ISA).
 __device__ __forceinline__ float rcp_fast(float d)
 {
     float r;

@@ -76,7 +76,8 @@ __device__ __forceinline__ void z_block(const float *col, int stride, const Coef
     }
 }
 
-// Approximate reciprocal of the damping factor 1 + s (normal: s lies in [0, 1) or so).
+// Approximate reciprocal of the damping factor 1 + s, a normal number near 1: rcp.approx.ftz is
+// within 1 ulp of the exact one (PTX ISA).
 __device__ __forceinline__ float rcp_damp(float d)
 {
     float r;
@@ -85,8 +86,7 @@ __device__ __forceinline__ float rcp_damp(float d)
 }
 
 // The damped update of a group: (2c + W lap - (1 - s) prev [+ srcv at point se]) / (1 + s),
-// packed; the quotient is the product with the approximate reciprocal, as __fdividef forms
-// it, without that function's scaling of divisors above 2^126.
+// packed; the quotient is the product with the approximate reciprocal of 1 + s.
 __device__ __forceinline__ float4 update4(float4 c, float2 l0, float2 l1, float4 pv, float4 Wv,
                                           float4 sx, float sz, int se, float srcv)
 {

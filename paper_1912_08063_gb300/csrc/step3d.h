@@ -212,18 +212,20 @@ cudaError_t launch_step2d_tile(const StepParams &p, int nshots, bool img, const 
 // cut over all CTAs; and S parts of which the first ones are longer and the leftover last parts
 // go to the CTAs that ran a last part.  It keeps the one whose busiest CTA streams the fewest
 // planes (warm-up planes included), the first one's weighed by (resident / CTAs used)^2 at
-// radius 8: its steps are bound by the SMs' instruction issue, and idle CTAs cost more there
-// (forward at 360^3, 552 of 608 CTAs and 106 planes 162.5 us, all CTAs and 115 planes 159.3; two
-// shots of 199 x 197 x 433, 546 CTAs and 83 planes 125, all and 95 planes 122; at 296^3, 570
-// and 66 planes 97, all and 79 planes 99).
-// Every launch of the step is planned in step.  Measured on GB300 (the radius-4 reverse step
-// still with two rows per thread), us per step forward /
+// radius 8: its steps are bound by the SMs' instruction issue, and idle CTAs cost more there.  Power
+// 0 / 1 / 2 of that weight on 11 grids of 216^3 to 440^3 computed points, us a step, where they differ
+// by more than 1 %: radius 8, 360^3 forward 162.4 / 157.6 / 157.8, store 182.5 / 175.7 / 175.6; two
+// shots of 199 x 197 x 433 forward 123.6 / 123.9 / 121.5, store 137.6 / 138.1 / 135.9.  Radius 4 takes
+// none: 296^3 reverse 109.0 / 112.5 / 112.4, 360^3 118.5 / 119.1 / 125.5 forward, 187.5 / 197.5 / 197.1
+// reverse, 440^3 forward 221.7 / 220.4 / 229.0.
+// Every launch of the step is planned in step.  Measured on GB300, us per step forward /
 // store / reverse, against one run of the columns cut over all CTAs below 96 MB and no
-// candidate without leftovers: radius 4, 216^3 39.2 / 45.5 / 69.6 -> 36.2 / 41.1 / 60.2, 280^3
-// 101 / 122 / 165 -> 63 / 72 / 109, 296^3 75.9 / 85.3 / 122 -> 70.7 / 81.5 / 122; radius 8, 240^3
-// 70 / 77 / 105 -> 55.6 / 61 / 71, 280^3 122 / 139 / 171 -> 86 / 95 / 102, 440^3 263 / 296 / 361 ->
-// 257 / 286 / 348.  Parts numbered column by column: radius 4 360^3 122 / 152 / 214 against
-// 119.6 / 137.8 / 212, 440^3 237 / 306 / 347 against 223 / 285 / 346.
+// candidate without leftovers: radius 4, 216^3 39.0 / 44.9 / 65.8 -> 35.9 / 40.8 / 54.2, 280^3
+// 99.9 / 117 / 159 -> 63.8 / 71.5 / 99.5, 296^3 74.9 / 84.6 / 112 -> 70.4 / 81.4 / 109; radius 8,
+// 216^3 60.5 / 68.0 / 85.3 -> 51.3 / 57.2 / 59.5, 280^3 120 / 135 / 169 -> 86.2 / 95.9 / 102, 440^3
+// 261 / 293 / 354 -> 255 / 287 / 344.  Parts numbered column by column (the reverse step then with
+// two rows per thread): radius 4 360^3 122 / 152 / 214 against 119.6 / 137.8 / 212, 440^3 237 / 306 /
+// 347 against 223 / 285 / 346.
 // Fills the schedule fields of p and returns the grid size.
 int plan_persistent(Step3dParams &p, int columns, int resident, bool in_step = false);
 

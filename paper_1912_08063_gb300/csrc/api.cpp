@@ -425,6 +425,23 @@ int64_t node_offset(const fwi_model *m, const int32_t *p)
 int ensure_workspace(fwi_model *m, const fwi_acq *a, bool grad, cudaStream_t s)
 {
     const int ns = a->nshots, nr = a->nrec;
+    const size_t nsrc = (size_t)ns * 3, nrec3 = (size_t)ns * nr * 3;
+    auto same_i = [](const std::vector<int32_t> &v, const int32_t *p, size_t n) {
+        return p ? (v.size() == n && std::memcmp(v.data(), p, n * sizeof(int32_t)) == 0)
+                 : v.empty();
+    };
+    auto same_d = [](const std::vector<double> &v, const double *p, size_t n) {
+        return p ? (v.size() == n && std::memcmp(v.data(), p, n * sizeof(double)) == 0)
+                 : v.empty();
+    };
+    const bool og_s = a->src_pos != nullptr, og_r = a->rec_pos != nullptr;
+    const bool same = m->geo_shots == ns && m->geo_nrec == nr &&
+                      (og_s ? same_d(m->geo_src_pos, a->src_pos, nsrc) : same_i(m->geo_src, a->src, nsrc)) &&
+                      (og_r ? same_d(m->geo_rec_pos, a->rec_pos, nrec3) : same_i(m->geo_rec, a->rec, nrec3)) &&
+                      m->og_src == og_s && m->og_rec == og_r;
+    // the tables are those of no geometry until they are complete: a call that fails on the way may
+    // have moved or overwritten some of them
+    if (!same) m->geo_shots = -1;
     const size_t fb = (size_t)m->g.field * sizeof(float);
     FWI_TRY(m->u[0].ensure(ns * fb));
     FWI_TRY(m->u[1].ensure(ns * fb));
@@ -444,20 +461,6 @@ int ensure_workspace(fwi_model *m, const fwi_acq *a, bool grad, cudaStream_t s)
     }
     if (ns > m->cap_shots) m->cap_shots = ns;
     if (nr > m->cap_nrec) m->cap_nrec = nr;
-    const size_t nsrc = (size_t)ns * 3, nrec3 = (size_t)ns * nr * 3;
-    auto same_i = [](const std::vector<int32_t> &v, const int32_t *p, size_t n) {
-        return p ? (v.size() == n && std::memcmp(v.data(), p, n * sizeof(int32_t)) == 0)
-                 : v.empty();
-    };
-    auto same_d = [](const std::vector<double> &v, const double *p, size_t n) {
-        return p ? (v.size() == n && std::memcmp(v.data(), p, n * sizeof(double)) == 0)
-                 : v.empty();
-    };
-    const bool og_s = a->src_pos != nullptr, og_r = a->rec_pos != nullptr;
-    bool same = m->geo_shots == ns && m->geo_nrec == nr &&
-                (og_s ? same_d(m->geo_src_pos, a->src_pos, nsrc) : same_i(m->geo_src, a->src, nsrc)) &&
-                (og_r ? same_d(m->geo_rec_pos, a->rec_pos, nrec3) : same_i(m->geo_rec, a->rec, nrec3)) &&
-                m->og_src == og_s && m->og_rec == og_r;
     if (!same) {
         std::vector<int64_t> so(ns, 0), ro((size_t)ns * nr, 0);
         if (og_s) {

@@ -59,6 +59,32 @@ def test_refused_launch_fails_its_own_call_only():
     m.close()
 
 
+def test_call_after_one_that_ran_out_of_memory():
+    """A call whose tap tables do not fit fails with FWI_ERR_OOM after it has replaced other tables;
+    the next call, with the geometry of the call before, builds its own again."""
+    from paper_1912_08063_gb300 import fwi
+    rng = np.random.default_rng(24)
+    v = torch.full((30, 40), 2000.0, device="cuda")
+    m = fwi.FwiModel(v, 10.0, 1e-3, 2)
+    wav = torch.ones(1, 2, device="cuda")
+    pos = lambda n: np.stack([rng.uniform(2, 28, n), np.zeros(n), rng.uniform(2, 38, n)], 1)   # noqa: E731
+    src = np.array([[15.0, 0, 20.0]])
+    acq = fwi.Acquisition(src_pos=src, rec_pos=src + [0.5, 0, 0.5])
+    before = m.forward(acq, wav)
+    big = fwi.Acquisition(src_pos=src, rec_pos=pos(4 << 20))    # 28 bytes a receiver, and 136 of taps
+    held = torch.empty(torch.cuda.mem_get_info()[0] - (400 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        with pytest.raises(fwi.FwiError) as e:
+            m.forward(big, wav, traces=torch.empty(1, 2, 4 << 20, device="cuda"))
+        assert e.value.code == fwi.FWI_ERR_OOM
+        after = m.forward(acq, wav)
+    finally:
+        del held
+        torch.cuda.empty_cache()
+    assert before.abs().max() > 0 and torch.equal(before, after)
+    m.close()
+
+
 def test_selftest_rejects_poll_limits_out_of_range():
     from paper_1912_08063_gb300 import fwi
     w, m = _small_model(fwi, np.random.default_rng(22))

@@ -76,9 +76,10 @@ constexpr int kWarps = 2, kMinCtas = 8;
 constexpr int kGridYMax = 65535;
 __host__ __device__ constexpr int tile_rz(int mode) { return mode == kImg ? 3 : 4; }
 
-// TAPS: an off-grid source is added too (an instantiation of its own, so that the common one
-// pays nothing for it: 3 % of a 64-shot step).
-template <int M, int MODE, bool TAPS>
+// TAPS: an off-grid source is added too.  MORE: the launch starts at tile row row0 (else 0).  Both
+// are instantiations of their own, so that the common one pays nothing for them (3 % and 0.5 % of a
+// 64-shot step).
+template <int M, int MODE, bool TAPS, bool MORE>
 __global__ void __launch_bounds__(32 * kWarps, kMinCtas)
 k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUtensorMap map, int row0)
 {
@@ -93,7 +94,7 @@ k_step2d_tile(const __grid_constant__ StepParams p, const __grid_constant__ CUte
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    const int tz = row0 + blockIdx.y;                           // tile row
+    const int tz = (MORE ? row0 : 0) + blockIdx.y;             // tile row
     const int x0 = blockIdx.x * kTileX + 4 * lane, zr = tz * TZ + warp * RZ;
     const bool xin = x0 < nx;
     const int plane = (int)p.g.plane;
@@ -263,13 +264,16 @@ template <int M, int MODE>
 cudaError_t go(const StepParams &p, int nshots, const CUtensorMap &map, cudaStream_t s)
 {
     constexpr int TZ = kWarps * tile_rz(MODE);
-    auto *fn = MODE != kImg && p.src_pts ? k_step2d_tile<M, MODE, MODE != kImg> : k_step2d_tile<M, MODE, false>;
+    auto *first = MODE != kImg && p.src_pts ? k_step2d_tile<M, MODE, MODE != kImg, false>
+                                            : k_step2d_tile<M, MODE, false, false>;
+    auto *more = MODE != kImg && p.src_pts ? k_step2d_tile<M, MODE, MODE != kImg, true>
+                                           : k_step2d_tile<M, MODE, false, true>;
     // tile rows on grid.y, at most 65535 a launch (a launch writes its own rows of prev only)
     const int rows = (p.g.nz + TZ - 1) / TZ;
     cudaError_t e = cudaSuccess;
     for (int row0 = 0; row0 < rows && e == cudaSuccess; row0 += kGridYMax) {
         const dim3 grid((p.g.nx + kTileX - 1) / kTileX, std::min(rows - row0, kGridYMax), nshots);
-        e = launch_pdl(fn, grid, dim3(32 * kWarps), 0, s, p, map, row0);
+        e = launch_pdl(row0 ? more : first, grid, dim3(32 * kWarps), 0, s, p, map, row0);
     }
     return e;
 }

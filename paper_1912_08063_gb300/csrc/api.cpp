@@ -2200,9 +2200,10 @@ void fwi_destroy(fwi_model *m)
 {
     if (!m) return;
     if (m->last_stream) cudaStreamSynchronize(m->last_stream);
-    if (m->h_flag) cudaFreeHost(m->h_flag);
     for (cudaEvent_t e : m->ev) cudaEventDestroy(e);
+    unsigned *flag = m->h_flag;   // kernels may write it until the buffers are freed
     delete m;
+    if (flag) cudaFreeHost(flag);
 }
 
 }  // extern "C"
